@@ -57,188 +57,438 @@ struct SiteSplit {
   float hx, lx, hy, ly, hz, lz, R, rin;
 };
 
-__device__ __forceinline__ bool pair_rule(const PairGrid& G, const PairTree& T, int64_t c, const SiteSplit& S,
-                                          int64_t k) {
-  const float* P = T.split + 6 * k;
-  const float fx = (P[0] - S.hx) + (P[1] - S.lx);
-  const float fy = (P[2] - S.hy) + (P[3] - S.ly);
-  const float fz = (P[4] - S.hz) + (P[5] - S.lz);
-  const float hf = T.hs32[k];
-  const float reach = fmaf(2.f, hf, S.R);
-  const float reach2 = reach * reach;
-  const float d2 = fx * fx + fy * fy + fz * fz;
-  if (d2 > reach2 * 1.00001f) return false;
-  if (!(d2 < reach2 * 0.99999f) &&
-      !exact_dist(G.site[3 * c], G.site[3 * c + 1], G.site[3 * c + 2], G.rad[c], T.xs[k], T.ys[k], T.zs[k], T.hs[k]))
-    return false;
-  const float thr = 2.f * hf;
+// The screens on the distance: outside (0), listed (1), or undecided (2).
+__device__ __forceinline__ int dist_screen(float d2, float reach2, float tin2) {
+  if (d2 > reach2 * 1.00001f) return 0;
   // every face test passes when the particle lies within 2h + r_in of the
   // site: each face plane is at least r_in from the site, so
   // n.r - d = n.(r - s) - (d - n.s) <= |r - s| - r_in < 2h for every face (the
   // 1e-4 relative margin covers the FP32 rounding many times over)
-  const float tin = thr + S.rin;
-  if (d2 < tin * tin * 0.9999f) return true;
-  const float l1 = fabsf(fx) + fabsf(fy) + fabsf(fz);
-  for (int64_t f = G.cfo[c]; f < G.cfo[c + 1]; ++f) {
-    const float4 F = G.face32[f];
-    const float sv = (F.x * fx + F.y * fy + F.z * fz) - F.w;
-    const float marg = 1e-5f * (l1 + fabsf(F.w) + thr) + 1e-30f;
-    if (sv > thr + marg) return false;
-    if (sv >= thr - marg && !exact_face(G.plane[f], T.xs[k], T.ys[k], T.zs[k], T.hs[k])) return false;
+  return d2 < fminf(reach2 * 0.99999f, tin2 * 0.9999f) ? 1 : 2;
+}
+
+// The rule for sorted position k; face(i) gives the cell's face record i of
+// nf (site-relative, FP32).
+template <typename F>
+__device__ __forceinline__ bool pair_rule(const PairGrid& G, const PairTree& T, int64_t c, int64_t f0, int nf,
+                                          const SiteSplit& S, int64_t k, F face) {
+  const float2* P = reinterpret_cast<const float2*>(T.split + 6 * k);
+  const float2 px = __ldg(P), py = __ldg(P + 1), pz = __ldg(P + 2);
+  const float fx = (px.x - S.hx) + (px.y - S.lx);
+  const float fy = (py.x - S.hy) + (py.y - S.ly);
+  const float fz = (pz.x - S.hz) + (pz.y - S.lz);
+  const float hf = __ldg(T.hs32 + k), thr = 2.f * hf;
+  const float reach = thr + S.R, tin = thr + S.rin;
+  const float reach2 = reach * reach;
+  const float d2 = fx * fx + fy * fy + fz * fz;
+  const int d = dist_screen(d2, reach2, tin * tin);
+  if (d < 2) return d == 1;
+  if (!(d2 < reach2 * 0.99999f) &&
+      !exact_dist(G.site[3 * c], G.site[3 * c + 1], G.site[3 * c + 2], G.rad[c], T.xs[k], T.ys[k], T.zs[k], T.hs[k]))
+    return false;
+  // the largest n.r - d over the faces, four at a time with their loads issued
+  // together (a chunk past the last face repeats it); |d - n.s| <= R for every
+  // face, so one margin covers them all
+  float smax = -INFINITY;
+  for (int f = 0; f < nf; f += 4) {
+    float4 Q[4];
+#pragma unroll
+    for (int i = 0; i < 4; ++i) Q[i] = face(f + i < nf ? f + i : nf - 1);
+#pragma unroll
+    for (int i = 0; i < 4; ++i) smax = fmaxf(smax, fmaf(Q[i].x, fx, fmaf(Q[i].y, fy, fmaf(Q[i].z, fz, -Q[i].w))));
   }
+  const float marg = 1e-5f * (fabsf(fx) + fabsf(fy) + fabsf(fz) + S.R + thr) + 1e-30f;
+  if (smax > thr + marg) return false;
+  if (smax >= thr - marg)
+    for (int f = 0; f < nf; ++f)
+      if (!exact_face(G.plane[f0 + f], T.xs[k], T.ys[k], T.zs[k], T.hs[k])) return false;
   return true;
+}
+__device__ __forceinline__ bool pair_rule(const PairGrid& G, const PairTree& T, int64_t c, const SiteSplit& S,
+                                          int64_t k) {
+  const int64_t f0 = G.cfo[c];
+  return pair_rule(G, T, c, f0, (int)(G.cfo[c + 1] - f0), S, k, [&](int i) { return __ldg(G.face32 + f0 + i); });
+}
+
+__device__ __forceinline__ SiteSplit site_split(const PairGrid& G, int64_t c) {
+  const double sx = G.site[3 * c], sy = G.site[3 * c + 1], sz = G.site[3 * c + 2];
+  SiteSplit S;
+  S.hx = (float)sx; S.lx = (float)(sx - (double)S.hx);
+  S.hy = (float)sy; S.ly = (float)(sy - (double)S.hy);
+  S.hz = (float)sz; S.lz = (float)(sz - (double)S.hz);
+  S.R = (float)G.rad[c];
+  S.rin = G.rin[c];
+  return S;
 }
 
 // One warp walks the octree for 32 cells that are consecutive in Morton order
-// of their sites (so close together), sharing the node loads: every lane
-// tests each visited node against its own cell (FP32, outward-rounded box,
-// 1e-6 absolute margin: 2 * largest h + cell radius) and the warp descends
-// when any lane needs the node.  At a leaf, the (cell, particle) tests of the
-// lanes that reach it are spread over all 32 lanes -- each lane's cell data
-// sit in shared memory -- and every hit is appended to its cell's list
-// (lanes with the same cell take consecutive places, in lane order).
-// FILL = false: count pairs per cell, keeping the first PAIR_ROW of them in
-// the cell's row of `out` (ncell x PAIR_ROW); FILL = true: write the pairs at
-// off[c] (the cells of `order` whose count exceeded the row; their number is
-// read from *n_dev).
+// of their sites (so close together), one cell per lane, depth-first, so that
+// the candidates come in sorted (Morton) order and each cell's list with them.
+//
+// Nodes: the lanes test a popped node's children side by side against the
+// box around the 32 sites; a child that survives is kept when any lane's own
+// cell can reach it (FP32, outward-rounded box, 1e-6 absolute margin:
+// 2 * largest h + cell radius).  Leaf children go on the stack as their
+// particle range, read with the box, so that nothing is loaded at the pop.
+//
+// Particles: the kept leaves' particles are staged 32 at a time in shared
+// memory (one load round for 32 candidates).  Every lane holds its cell in
+// registers and classifies all 32 against it by the distance alone: outside,
+// listed for certain (within 2h + r_in of the site), or undecided.
+//
+// WALK_ROWS: both kinds go to the cell's row in HBM as sorted positions, the
+// undecided ones (half of them) marked; row_filter then settles those with
+// one warp per cell.  A row holds PAIR_ROW entries; a longer one goes on in
+// chunks of a pool (1% of the clumpy cells; the pool holds two chunks per cell
+// of a small grid, 1/32 per cell beyond 2048), and a cell that finds the pool
+// empty is put on the list `again`.
+// WALK_COUNT / WALK_FILL: for the cells of that list, the rule is settled here
+// (the undecided tests of the warp compacted over its lanes) and the pairs
+// counted, or written at off[c].
+//
+// What bounds it: the chain of one warp, about 1000 candidates classified at
+// 20 instructions for 32 cells.  At 2^20 clumpy cells the walk takes 3.4 ms
+// and the filter 2.3 ms; at 60,000 the whole pair list takes 0.73 ms.  Testing
+// leaf by leaf, the (cell, particle) tests of the reaching lanes spread over
+// the warp, waited for the loads of every test: 12.7 ms, and 2.1 ms at 60,000,
+// where a warp's chain is the whole time.  Settling the undecided tests inside
+// the walk took half of its 6.2 and 0.77 ms.
 constexpr int PAIR_ROW = 256;
-constexpr int PT_WARPS = 4;  // warps per block of the traversal (1 and 2 measured: no faster)
-// CTAs per SM the traversal is compiled for: 12 caps it at 40 registers (a
-// few spilled) for 48 resident warps; the walk waits on its node and
-// candidate loads, so the extra warps pay (2^20: 15.2 ms at 64 registers,
-// 14.0 at 48, 13.6 at 40, 16.1 at 32)
-constexpr int PT_MINB = 12;
+constexpr int PT_WARPS = 4;   // warps per block of the traversal
+constexpr int PT_STK = 160;   // a popped node pushes at most 8 children; 22 levels at most: 155 entries
+enum { WALK_ROWS, WALK_COUNT, WALK_FILL };
 
-struct WalkCells {  // per warp: the 32 lanes' cells, one entry per lane
-  float hx[32], lx[32], hy[32], ly[32], hz[32], lz[32], R[32], rin[32];
-  int64_t c[32], w[32], cnt[32];
-  int32_t need[32];  // the lanes that reach the current leaf, in lane order
+// Rows of candidates: rows[c * PAIR_ROW ...], then chunks of a pool.
+struct PairRows {
+  int32_t* rows;
+  int32_t* pool;              // npool chunks of PAIR_ROW entries
+  int32_t* first;             // per cell: its first chunk (-1: none; -2: the pool was empty)
+  int32_t* next;              // per chunk: the cell's next one
+  int32_t npool;
+  unsigned long long* used;   // chunks handed out
+  int32_t* again;             // the cells that found none left
+  unsigned long long* n_again;
 };
 
-template <bool FILL>
-__global__ void __launch_bounds__(PT_WARPS * 32, PT_MINB)
+// FP32 pairs in one instruction
+struct f2 { float x, y; };
+__device__ __forceinline__ unsigned long long f2_bits(f2 a) {
+  return (unsigned long long)__float_as_uint(a.x) | ((unsigned long long)__float_as_uint(a.y) << 32);
+}
+__device__ __forceinline__ f2 f2_from(unsigned long long b) {
+  return f2{__uint_as_float((unsigned)b), __uint_as_float((unsigned)(b >> 32))};
+}
+__device__ __forceinline__ f2 add2(f2 a, f2 b) {
+  unsigned long long d;
+  asm("add.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(f2_bits(a)), "l"(f2_bits(b)));
+  return f2_from(d);
+}
+__device__ __forceinline__ f2 mul2(f2 a, f2 b) {
+  unsigned long long d;
+  asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(f2_bits(a)), "l"(f2_bits(b)));
+  return f2_from(d);
+}
+
+struct WalkWarp {
+  int2 stk[PT_STK];       // internal node: (first child, children); leaf: (first position, -particles)
+  float4 ca[32], cb[32];  // staged candidates: (x hi, y hi, x lo, y lo), (z hi, 2h, z lo, -)
+  int32_t k[64];          // sorted positions of the candidates gathered
+  float4 ba[8], bb[8];    // the popped node's children: boxes and links
+};
+struct WalkExact {              // WALK_COUNT, WALK_FILL
+  float4 sa[32], sb[32];        // the lanes' cells: (x hi, lo, y hi, lo), (z hi, lo, R, r_in)
+  unsigned rej[32];             // undecided tests that failed
+  unsigned short und[32 * 32];  // undecided tests: cell lane << 5 | candidate
+};
+
+template <int MODE>
+__global__ void __launch_bounds__(PT_WARPS * 32)
     pair_traverse(int64_t ncell, const int32_t* __restrict__ order, PairTree T, PairGrid G, int64_t* count,
-                  const int64_t* __restrict__ off, int32_t* out, const unsigned long long* n_dev,
-                  int64_t cap = INT64_MAX) {
-  __shared__ int32_t s_stack[PT_WARPS][200];
-  if (FILL && off[ncell] > cap) return;  // the list does not fit its buffer: nothing is written
-  __shared__ WalkCells s_cells[PT_WARPS];
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+                  PairRows Q, const int64_t* __restrict__ off, int32_t* out, int64_t cap) {
+  constexpr bool EXACT = MODE != WALK_ROWS;
+  __shared__ WalkWarp s_walk[PT_WARPS];
+  __shared__ WalkExact s_exact[EXACT ? PT_WARPS : 1];
+  if (MODE == WALK_FILL && off[ncell] > cap) return;  // the list does not fit its buffer: nothing is written
+  constexpr unsigned FULL = 0xffffffffu;
+  const int lane = threadIdx.x & 31;
   const unsigned lt = (1u << lane) - 1u;
+  WalkWarp& W = s_walk[threadIdx.x >> 5];
+  WalkExact& X = s_exact[EXACT ? threadIdx.x >> 5 : 0];
   const int64_t t = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x);
-  const bool valid = t < (n_dev ? (int64_t)*n_dev : ncell);
-  if (__all_sync(0xffffffffu, !valid)) return;
-  const int64_t c = valid ? (order ? order[t] : t) : -1;
-  double sx = 0, sy = 0, sz = 0, R = 0;
-  if (valid) { sx = G.site[3 * c]; sy = G.site[3 * c + 1]; sz = G.site[3 * c + 2]; R = G.rad[c]; }
-  const float fsx = (float)sx, fsy = (float)sy, fsz = (float)sz, fR = (float)R;
-  WalkCells& W = s_cells[warp];
-  W.hx[lane] = fsx; W.lx[lane] = (float)(sx - (double)fsx);
-  W.hy[lane] = fsy; W.ly[lane] = (float)(sy - (double)fsy);
-  W.hz[lane] = fsz; W.lz[lane] = (float)(sz - (double)fsz);
-  W.R[lane] = fR;
-  W.rin[lane] = valid ? G.rin[c] : 0.f;
-  W.c[lane] = c;
-  W.w[lane] = valid ? (FILL ? off[c] : c * PAIR_ROW) : 0;
-  W.cnt[lane] = 0;
-  int32_t* stack = s_stack[warp];
-  int sp = 1;
-  if (lane == 0) stack[0] = 0;
+  const bool valid = t < (EXACT ? (int64_t)*Q.n_again : ncell);
+  if (!__any_sync(FULL, valid)) return;
+  const int64_t c = valid ? (EXACT ? Q.again[t] : order[t]) : -1;
+  SiteSplit SS{};
+  if (valid) SS = site_split(G, c);
+  const float hx = SS.hx, hy = SS.hy, hz = SS.hz, fR = SS.R, rin = SS.rin;
+  if (EXACT) {
+    X.sa[lane] = make_float4(hx, SS.lx, hy, SS.ly);
+    X.sb[lane] = make_float4(hz, SS.lz, fR, rin);
+  }
+  // the box around the warp's sites and the largest cell radius
+  float gx0 = valid ? hx : INFINITY, gx1 = valid ? hx : -INFINITY, gy0 = valid ? hy : INFINITY;
+  float gy1 = valid ? hy : -INFINITY, gz0 = valid ? hz : INFINITY, gz1 = valid ? hz : -INFINITY, gR = fR;
+  for (int o = 16; o > 0; o >>= 1) {
+    gx0 = fminf(gx0, __shfl_xor_sync(FULL, gx0, o)); gx1 = fmaxf(gx1, __shfl_xor_sync(FULL, gx1, o));
+    gy0 = fminf(gy0, __shfl_xor_sync(FULL, gy0, o)); gy1 = fmaxf(gy1, __shfl_xor_sync(FULL, gy1, o));
+    gz0 = fminf(gz0, __shfl_xor_sync(FULL, gz0, o)); gz1 = fmaxf(gz1, __shfl_xor_sync(FULL, gz1, o));
+    gR = fmaxf(gR, __shfl_xor_sync(FULL, gR, o));
+  }
+  int32_t* row = nullptr;  // where the next entry goes
+  int left = INT32_MAX;    // entries that fit there
+  int chunk = -1;          // the chunk it lies in (-1: the row itself; -2: no chunk was left)
+  if (valid && MODE == WALK_ROWS) { row = Q.rows + c * PAIR_ROW; left = PAIR_ROW; Q.first[c] = -1; }
+  if (valid && MODE == WALK_FILL) row = out + off[c];
+  int cnt = 0;
+  int nk = 0;  // candidates gathered (warp-uniform)
+
+  // the first n (<= 32) candidates gathered against the 32 cells
+  auto test = [&](int n) {
+    __syncwarp();
+    if (lane < n) {
+      const int64_t k = W.k[lane];
+      const float2* P = reinterpret_cast<const float2*>(T.split + 6 * k);
+      const float2 px = __ldg(P), py = __ldg(P + 1), pz = __ldg(P + 2);
+      W.ca[lane] = make_float4(px.x, py.x, px.y, py.y);
+      W.cb[lane] = make_float4(pz.x, 2.f * __ldg(T.hs32 + k), pz.y, 0.f);
+    }
+    if (EXACT) X.rej[lane] = 0u;
+    __syncwarp();
+    unsigned acc = 0u, und = 0u;  // listed for certain, undecided
+#pragma unroll 4
+    for (int j = 0; j < n; ++j) {
+      const float4 A = W.ca[j], B = W.cb[j];
+      // in two-lane arithmetic: (x, y) of the offset; (z hi, reach), (z lo, 2h + r_in)
+      const f2 e = add2(add2(f2{A.x, A.y}, f2{-hx, -hy}), add2(f2{A.z, A.w}, f2{-SS.lx, -SS.ly}));
+      const f2 u = add2(f2{B.x, B.y}, f2{-hz, fR}), v = add2(f2{B.z, B.y}, f2{-SS.lz, rin});
+      const float fz = u.x + v.x;
+      const float d2 = fmaf(e.x, e.x, fmaf(e.y, e.y, fz * fz));
+      const f2 r2 = mul2(f2{u.y, v.y}, f2{u.y, v.y});
+      const int s = dist_screen(d2, r2.x, r2.y);
+      acc |= (unsigned)(s == 1) << j;
+      und |= (unsigned)(s == 2) << j;
+    }
+    if (!valid) acc = und = 0u;
+    if (!EXACT) {
+      for (unsigned m = acc | und; m; m &= m - 1u) {
+        const int j = __ffs(m) - 1;
+        ++cnt;
+        if (left == 0) {
+          const unsigned long long q = chunk != -2 ? atomicAdd(Q.used, 1ULL) : ~0ULL;
+          if (q >= (unsigned long long)Q.npool) { chunk = -2; continue; }
+          if (chunk < 0) Q.first[c] = (int32_t)q; else Q.next[chunk] = (int32_t)q;
+          chunk = (int)q;
+          row = Q.pool + (int64_t)chunk * PAIR_ROW;
+          left = PAIR_ROW;
+        }
+        *row++ = W.k[j] | (int32_t)((und >> j & 1u) << 31);
+        --left;
+      }
+      return;
+    }
+    const int nu = __popc(und);
+    int o = nu;
+#pragma unroll
+    for (int d = 1; d < 32; d <<= 1) {
+      const int v = __shfl_up_sync(FULL, o, d);
+      if (lane >= d) o += v;
+    }
+    const int U = __shfl_sync(FULL, o, 31);
+    o -= nu;
+    for (unsigned m = und; m; m &= m - 1u) X.und[o++] = (unsigned short)(lane << 5 | (__ffs(m) - 1));
+    __syncwarp();
+    for (int r = 0; r < U; r += 32) {
+      const bool on = r + lane < U;
+      const int e = X.und[on ? r + lane : r];
+      const int l = e >> 5, j = e & 31;
+      const int64_t cl = __shfl_sync(FULL, c, l);
+      if (on) {
+        const float4 a = X.sa[l], b = X.sb[l];
+        if (!pair_rule(G, T, cl, SiteSplit{a.x, a.y, a.z, a.w, b.x, b.y, b.z, b.w}, W.k[j])) atomicOr(&X.rej[l], 1u << j);
+      }
+    }
+    __syncwarp();
+    acc |= und & ~X.rej[lane];
+    if (MODE == WALK_FILL)
+      for (unsigned m = acc; m; m &= m - 1u) *row++ = T.idx[W.k[__ffs(m) - 1]];
+    cnt += __popc(acc);
+  };
+  // particles [a, a + k) join the candidates; full rounds of 32 are tested
+  auto gather = [&](int a, int k) {
+    while (k > 0) {
+      const int g = k < 32 ? k : 32;
+      if (lane < g) W.k[nk + lane] = a + lane;
+      nk += g;
+      a += g;
+      k -= g;
+      if (nk >= 32) {
+        test(32);
+        nk -= 32;
+        __syncwarp();
+        const int32_t v = lane < nk ? W.k[32 + lane] : 0;
+        __syncwarp();
+        if (lane < nk) W.k[lane] = v;
+      }
+    }
+  };
+
+  int sp = 0;
+  const int nroot = T.nch[0];
+  if (nroot == 0) {
+    gather((int)T.nb[0], (int)(T.ne[0] - T.nb[0]));  // the root is a leaf
+  } else {
+    if (lane == 0) W.stk[0] = make_int2((int)T.fc[0], nroot);
+    sp = 1;
+  }
   __syncwarp();
   while (sp > 0) {
-    const int32_t nd = stack[--sp];
+    const int2 E = W.stk[--sp];
     __syncwarp();
-    const float4 b0 = reinterpret_cast<const float4*>(T.box32)[2 * (int64_t)nd];
-    const float4 b1 = reinterpret_cast<const float4*>(T.box32)[2 * (int64_t)nd + 1];
-    const float dx = fsx < b0.x ? b0.x - fsx : (fsx > b0.w ? fsx - b0.w : 0.f);
-    const float dy = fsy < b0.y ? b0.y - fsy : (fsy > b1.x ? fsy - b1.x : 0.f);
-    const float dz = fsz < b0.z ? b0.z - fsz : (fsz > b1.y ? fsz - b1.y : 0.f);
-    const float reach = (2.f * b1.z + fR + 1e-6f) * 1.000001f;
-    const bool need = valid && dx * dx + dy * dy + dz * dz <= reach * reach;
-    const unsigned mneed = __ballot_sync(0xffffffffu, need);
-    if (!mneed) continue;
-    const unsigned link = __float_as_uint(b1.w);
-    if (link == 0u) {
-      const int64_t k0 = T.nb[nd];
-      const int nl = (int)(T.ne[nd] - k0);
-      const int nn = __popc(mneed);
-      if (need) W.need[__popc(mneed & lt)] = lane;
-      __syncwarp();
-      // tests (needing cell i, particle j): chunks of up to 32 particles, g
-      // cells per round, lane -> (i = r + lane / chunk, j = p + lane % chunk)
-      const int chunk = nl < 32 ? nl : 32;
-      const int g = chunk > 0 ? 32 / chunk : 1;
-      const int li = chunk > 0 ? lane / chunk : 0, lj = chunk > 0 ? lane - li * chunk : 0;
-      for (int p = 0; p < nl; p += chunk) {
-        for (int r = 0; r < nn; r += g) {
-          const int i = r + li, j = p + lj;
-          const bool on = li < g && i < nn && j < nl;
-          const int l = on ? W.need[i] : 0;
-          bool hit = false;
-          if (on) {
-            SiteSplit SS;
-            SS.hx = W.hx[l]; SS.lx = W.lx[l];
-            SS.hy = W.hy[l]; SS.ly = W.ly[l];
-            SS.hz = W.hz[l]; SS.lz = W.lz[l];
-            SS.R = W.R[l];
-            SS.rin = W.rin[l];
-            hit = pair_rule(G, T, W.c[l], SS, k0 + j);
-          }
-          if (__any_sync(0xffffffffu, hit)) {
-            const unsigned grp = __match_any_sync(0xffffffffu, hit ? l : 32 + lane);
-            int64_t q = 0;
-            if (hit) {
-              q = W.cnt[l] + __popc(grp & lt);
-              if (FILL || q < PAIR_ROW) out[W.w[l] + q] = T.idx[k0 + j];
-            }
-            __syncwarp();
-            if (hit && (grp & lt) == 0) W.cnt[l] += __popc(grp);
-            __syncwarp();
-          }
+    if (E.y < 0) {
+      gather(E.x, -E.y);
+      continue;
+    }
+    bool near = false;
+    int2 mine = make_int2(0, 0);
+    if (lane < E.y) {
+      const int64_t nd = (int64_t)E.x + lane;
+      const float4 b0 = __ldg(reinterpret_cast<const float4*>(T.box32) + 2 * nd);
+      const float4 b1 = __ldg(reinterpret_cast<const float4*>(T.box32) + 2 * nd + 1);
+      const float dx = fmaxf(fmaxf(b0.x - gx1, gx0 - b0.w), 0.f);
+      const float dy = fmaxf(fmaxf(b0.y - gy1, gy0 - b1.x), 0.f);
+      const float dz = fmaxf(fmaxf(b0.z - gz1, gz0 - b1.y), 0.f);
+      const float reach = (2.f * b1.z + gR + 1e-6f) * 1.00001f;
+      near = dx * dx + dy * dy + dz * dz <= reach * reach;
+      if (near) {
+        W.ba[lane] = b0;
+        W.bb[lane] = b1;
+        const unsigned link = __float_as_uint(b1.w);
+        if (link == 0u) {
+          const int64_t a = T.nb[nd];
+          mine = make_int2((int)a, -(int)(T.ne[nd] - a));
+        } else if (link == NODE_LINK_FAR) {
+          mine = make_int2((int)T.fc[nd], T.nch[nd]);
+        } else {
+          mine = make_int2((int)(link >> 4), (int)(link & 15u));
         }
       }
-    } else {
-      const int nc = link == NODE_LINK_FAR ? T.nch[nd] : (int)(link & 15u);
-      const int64_t c0 = link == NODE_LINK_FAR ? T.fc[nd] : (int64_t)(link >> 4);
-      if (lane < nc) stack[sp + lane] = (int32_t)(c0 + nc - 1 - lane);
-      sp += nc;
-      __syncwarp();
+    }
+    unsigned m = __ballot_sync(FULL, near);
+    __syncwarp();
+    unsigned keep = 0u;
+    for (; m; m &= m - 1u) {
+      const int i = __ffs(m) - 1;
+      const float4 b0 = W.ba[i], b1 = W.bb[i];
+      const float dx = fmaxf(fmaxf(b0.x - hx, hx - b0.w), 0.f);
+      const float dy = fmaxf(fmaxf(b0.y - hy, hy - b1.x), 0.f);
+      const float dz = fmaxf(fmaxf(b0.z - hz, hz - b1.y), 0.f);
+      const float reach = (2.f * b1.z + fR + 1e-6f) * 1.000001f;
+      if (__any_sync(FULL, valid && dx * dx + dy * dy + dz * dz <= reach * reach)) keep |= 1u << i;
+    }
+    // pushed last child first, so that they pop in child order
+    const int nkeep = __popc(keep);
+    if (sp + nkeep > PT_STK) break;  // unreachable for trees of at most 22 levels
+    if (keep >> lane & 1u) W.stk[sp + nkeep - 1 - __popc(keep & lt)] = mine;
+    sp += nkeep;
+    __syncwarp();
+  }
+  if (nk > 0) test(nk);
+  if (valid && MODE != WALK_FILL) {
+    count[c] = cnt;
+    if (MODE == WALK_ROWS && chunk == -2) {
+      Q.first[c] = -2;
+      Q.again[atomicAdd(Q.n_again, 1ULL)] = (int32_t)c;
     }
   }
-  if (!FILL && valid) count[c] = W.cnt[lane];
+}
+
+// Settles the undecided entries of a cell's row, one warp per cell: its faces
+// go to shared memory in one load, its entries come 32 at a time, and the row
+// is packed in place (the writes stay behind the reads) as particle indices;
+// count[c] becomes the number of pairs.  Bound by the gathers of the entries'
+// positions.
+constexpr int RF_FACES = 64;  // faces staged; a cell with more reads them from global memory
+__global__ void __launch_bounds__(128, 10) row_filter(int64_t ncell, const int32_t* __restrict__ order, PairTree T,
+                                                  PairGrid G, PairRows Q, int64_t* count) {
+  __shared__ float4 s_face[4][RF_FACES];
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int64_t t = blockIdx.x * 4LL + warp;
+  if (t >= ncell) return;  // whole warp
+  const int64_t c = order[t];
+  const int link = Q.first[c];
+  if (link == -2) return;  // walked again
+  const int n = (int)count[c];
+  const int64_t f0 = G.cfo[c];
+  const int nf = (int)(G.cfo[c + 1] - f0);
+  float4* sf = s_face[warp];
+  const bool staged = nf <= RF_FACES;
+  if (staged)
+    for (int i = lane; i < nf; i += 32) sf[i] = __ldg(G.face32 + f0 + i);
+  const SiteSplit SS = site_split(G, c);
+  __syncwarp();
+  int32_t* rp = Q.rows + c * PAIR_ROW;  // the part read, the part written
+  int32_t* wp = rp;
+  int rnext = link, wnext = link;       // the chunks that follow them
+  int w = 0;                            // entries in the part written
+  int64_t hits = 0;
+  for (int b = 0; b < n; b += 32) {
+    if (b > 0 && b % PAIR_ROW == 0) {
+      rp = Q.pool + (int64_t)rnext * PAIR_ROW;
+      rnext = Q.next[rnext];  // (of the last chunk: never followed)
+    }
+    bool pass = b + lane < n;
+    int64_t k = 0;
+    if (pass) {
+      const int32_t e = rp[b % PAIR_ROW + lane];
+      k = e & 0x7fffffff;
+      if (e < 0)
+        pass = staged ? pair_rule(G, T, c, f0, nf, SS, k, [&](int i) { return sf[i]; })
+                      : pair_rule(G, T, c, f0, nf, SS, k, [&](int i) { return __ldg(G.face32 + f0 + i); });
+    }
+    const unsigned m = __ballot_sync(0xffffffffu, pass);
+    const int at = w + __popc(m & ((1u << lane) - 1u));
+    int32_t* np = w + __popc(m) > PAIR_ROW ? Q.pool + (int64_t)wnext * PAIR_ROW : nullptr;
+    if (pass) {
+      const int32_t a = T.idx[k];
+      if (at < PAIR_ROW) wp[at] = a; else np[at - PAIR_ROW] = a;
+    }
+    w += __popc(m);
+    hits += __popc(m);
+    if (np) {
+      wp = np;
+      wnext = Q.next[wnext];
+      w -= PAIR_ROW;
+    }
+    __syncwarp();
+  }
+  if (lane == 0) count[c] = hits;
 }
 
 // The same walk with one warp per cell, for grids with many particles per
 // cell (few, large cells): lanes test a node's children in parallel, the
 // particles of the leaves the cell reaches are gathered in a buffer, and all
-// 32 lanes apply the pair rule to 32 candidates at a time.  Output as
-// pair_traverse (any order: each cell's list is sorted afterwards).
+// 32 lanes apply the pair rule to 32 candidates at a time.  FILL = false:
+// count pairs per cell, keeping the first PAIR_ROW of them in the cell's row;
+// FILL = true: write the pairs of the cells `again` at off[c].
 constexpr int WALK_STK = 160;   // a popped node pushes at most 8 of its children; 22 levels at most
 constexpr int WALK_CAND = 512;  // candidate positions gathered before they are tested
 
 template <bool FILL>
-__global__ void __launch_bounds__(128) pair_walk_warp(int64_t ncell, const int32_t* __restrict__ cells, PairTree T,
-                                                      PairGrid G, int64_t* count, const int64_t* __restrict__ off,
-                                                      int32_t* out, const unsigned long long* n_dev,
-                                                      int64_t cap = INT64_MAX) {
+__global__ void __launch_bounds__(128) pair_walk_warp(int64_t ncell, PairTree T, PairGrid G, int64_t* count,
+                                                      PairRows Q, const int64_t* __restrict__ off, int32_t* list,
+                                                      int64_t cap) {
   __shared__ int32_t s_stk[4][WALK_STK];
   if (FILL && off[ncell] > cap) return;  // the list does not fit its buffer: nothing is written
   __shared__ int32_t s_cand[4][WALK_CAND];
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int64_t t = blockIdx.x * 4 + warp;
-  if (t >= (n_dev ? (int64_t)*n_dev : ncell)) return;  // whole warp
-  const int64_t c = cells ? cells[t] : t;
-  const double sx = G.site[3 * c], sy = G.site[3 * c + 1], sz = G.site[3 * c + 2], R = G.rad[c];
-  const float fsx = (float)sx, fsy = (float)sy, fsz = (float)sz, fR = (float)R;
-  SiteSplit SS;
-  SS.hx = fsx; SS.lx = (float)(sx - (double)fsx);
-  SS.hy = fsy; SS.ly = (float)(sy - (double)fsy);
-  SS.hz = fsz; SS.lz = (float)(sz - (double)fsz);
-  SS.R = fR;
-  SS.rin = G.rin[c];
+  if (t >= (FILL ? (int64_t)*Q.n_again : ncell)) return;  // whole warp
+  const int64_t c = FILL ? Q.again[t] : t;
+  const SiteSplit SS = site_split(G, c);
+  const float fsx = SS.hx, fsy = SS.hy, fsz = SS.hz, fR = SS.R;
   int32_t* stk = s_stk[warp];
   int32_t* cand = s_cand[warp];
-  int64_t w = FILL ? off[c] : c * PAIR_ROW;
+  int32_t* const out = FILL ? list + off[c] : Q.rows + c * PAIR_ROW;
   int64_t cnt = 0;
   int sp = 1, nc_ = 0;  // stack depth, candidates held
   if (lane == 0) stk[0] = 0;
@@ -252,7 +502,7 @@ __global__ void __launch_bounds__(128) pair_walk_warp(int64_t ncell, const int32
       const unsigned m = __ballot_sync(0xffffffffu, hit);
       if (hit) {
         const int64_t q = cnt + __popc(m & ((1u << lane) - 1u));
-        if (FILL || q < PAIR_ROW) out[w + q] = T.idx[cand[j]];
+        if (FILL || q < PAIR_ROW) out[q] = T.idx[cand[j]];
       }
       cnt += __popc(m);
     }
@@ -313,24 +563,35 @@ __global__ void __launch_bounds__(128) pair_walk_warp(int64_t ncell, const int32
   if (!FILL && lane == 0) count[c] = cnt;
 }
 
-// Move the rows kept by the counting pass to their place in the list (one
-// warp per cell); cells whose count exceeded the row go to the overflow list
-// for the filling pass.
+// Move the rows to their place in the list (one warp per cell).
 __global__ void __launch_bounds__(128) place_rows(int64_t ncell, const int64_t* __restrict__ count,
-                                                  const int64_t* __restrict__ off, const int32_t* __restrict__ rows,
-                                                  int32_t* out, int32_t* ovf, unsigned long long* n_ovf,
-                                                  int64_t cap = INT64_MAX) {
+                                                  const int64_t* __restrict__ off, PairRows Q, int32_t* out,
+                                                  int64_t cap) {
   const int64_t c = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5;
   const int lane = threadIdx.x & 31;
   if (c >= ncell || off[ncell] > cap) return;
+  int q = Q.first[c];
+  if (q == -2) return;  // written by the second walk
   const int64_t n = count[c];
-  if (n > PAIR_ROW) {
-    if (lane == 0) ovf[atomicAdd(n_ovf, 1ULL)] = (int32_t)c;
-    return;
-  }
-  const int32_t* src = rows + c * PAIR_ROW;
+  const int32_t* src = Q.rows + c * PAIR_ROW;
   int32_t* dst = out + off[c];
-  for (int64_t i = lane; i < n; i += 32) dst[i] = src[i];
+  for (int64_t b = 0; b < n; b += PAIR_ROW) {
+    const int m = (int)(n - b < PAIR_ROW ? n - b : PAIR_ROW);
+    for (int i = lane; i < m; i += 32) dst[b + i] = src[i];
+    if (n - b <= PAIR_ROW) break;
+    src = Q.pool + (int64_t)q * PAIR_ROW;
+    q = Q.next[q];
+  }
+}
+
+// The cells of pair_walk_warp whose pairs outnumber their row (no chunks
+// there): first[c] and the list of cells to walk again.
+__global__ void mark_again(int64_t ncell, const int64_t* __restrict__ count, PairRows Q) {
+  const int64_t c = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+  if (c >= ncell) return;
+  const bool over = count[c] > PAIR_ROW;
+  Q.first[c] = over ? -2 : -1;
+  if (over) Q.again[atomicAdd(Q.n_again, 1ULL)] = (int32_t)c;
 }
 
 // Work items: cell c's n pairs in max(1, ceil(ceil(n/32)/K)) items of at
@@ -412,16 +673,16 @@ __global__ void mark_large(int64_t ncell, const int64_t* __restrict__ off, int64
   }
 }
 
-__global__ void site_keys(int64_t n, const double* __restrict__ site, uint64_t* keys, int32_t* idx) {
+__global__ void site_keys(int64_t n, const double* __restrict__ site, uint32_t* keys, int32_t* idx) {
   int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
   if (i >= n) return;
-  auto q = [](double v) -> uint64_t {
+  auto q = [](double v) -> uint32_t {
     double s = floor(v * 1024.0);
     s = s < 0 ? 0 : (s > 1023 ? 1023 : s);
-    return (uint64_t)s;
+    return (uint32_t)s;
   };
-  uint64_t k = 0;
-  uint64_t xi = q(site[3 * i]), yi = q(site[3 * i + 1]), zi = q(site[3 * i + 2]);
+  uint32_t k = 0;
+  uint32_t xi = q(site[3 * i]), yi = q(site[3 * i + 1]), zi = q(site[3 * i + 2]);
   for (int b = 9; b >= 0; --b) k = (k << 3) | (((xi >> b) & 1) << 2) | (((yi >> b) & 1) << 1) | ((zi >> b) & 1);
   keys[i] = k;
   idx[i] = (int32_t)i;
@@ -430,42 +691,102 @@ __global__ void site_keys(int64_t n, const double* __restrict__ site, uint64_t* 
 
 }  // namespace
 
-int pairs_build(map_ctx* ctx, const PreparedGrid* g, cudaStream_t s, const PairBufs& out) {
+namespace {
+
+// A pair-list build's launches, shared by the build that reads its sizes back
+// and the one that does not.
+struct PairWalk {
+  PairTree T;
+  PairGrid G;
+  PairRows Q;
+  int32_t* order;
+  int64_t* count;
+  bool per_warp;
+};
+
+// Every cell's pairs in its row (or on the list of cells to walk again), and
+// their counts.
+int walk_rows(map_ctx* ctx, const PreparedGrid* g, cudaStream_t s, PairWalk& P) {
   DevTree& T = ctx->tree;
   const int64_t nc = g->ncell;
   const int tpb = 128;
   // cells visited in Morton order of their sites for coherent traversals
-  uint64_t *k_in, *k_out;
-  int32_t *o_in, *order;
+  uint32_t *k_in, *k_out;
+  int32_t* o_in;
   MAP_TRY(ensure_t(ctx, ctx->ws_pairs[4], nc, &k_in));
   MAP_TRY(ensure_t(ctx, ctx->ws_pairs[5], nc, &k_out));
   MAP_TRY(ensure_t(ctx, ctx->ws_pairs[6], nc, &o_in));
-  MAP_TRY(ensure_t(ctx, ctx->ws_pairs[14], nc, &order));  // kept for the inverse mapping's gather order
+  MAP_TRY(ensure_t(ctx, ctx->ws_pairs[14], nc, &P.order));  // kept for the inverse mapping's gather order
   site_keys<<<nblk(nc, 256), 256, 0, s>>>(nc, g->site, k_in, o_in); ++ctx->launches;
   CUDA_TRY(cudaGetLastError());
   size_t tb = 0;
-  CUDA_TRY(cub::DeviceRadixSort::SortPairs(nullptr, tb, k_in, k_out, o_in, order, nc, 0, 30, s));
+  CUDA_TRY(cub::DeviceRadixSort::SortPairs(nullptr, tb, k_in, k_out, o_in, P.order, nc, 0, 30, s));
   MAP_TRY(ctx_ensure(ctx, ctx->cub_tmp, tb));
-  CUDA_TRY(cub::DeviceRadixSort::SortPairs(ctx->cub_tmp.p, tb, k_in, k_out, o_in, order, nc, 0, 30, s));
+  CUDA_TRY(cub::DeviceRadixSort::SortPairs(ctx->cub_tmp.p, tb, k_in, k_out, o_in, P.order, nc, 0, 30, s));
 
-  PairTree PT{T.xs, T.ys, T.zs, T.hs, T.hs32, T.split, T.idx, T.begin, T.end, T.first_child, T.nchild, T.bbox_bits,
-              T.hmax_bits, T.box32};
-  PairGrid PG{g->cell_face_off, g->face_plane, g->face32, g->site, g->rad, g->rin};
-  int64_t *count, *off;
-  MAP_TRY(ensure_t(ctx, ctx->ws_pairs[0], nc + 1, &count));
-  MAP_TRY(ensure_t(ctx, out.off ? *out.off : ctx->ws_pairs[1], nc + 1, &off));
-  int32_t* rows;
-  MAP_TRY(ensure_t(ctx, ctx->ws_pairs[8], (size_t)nc * PAIR_ROW, &rows));
-  CUDA_TRY(cudaMemsetAsync(count + nc, 0, sizeof(int64_t), s));
+  P.T = PairTree{T.xs, T.ys, T.zs, T.hs, T.hs32, T.split, T.idx, T.begin, T.end, T.first_child, T.nchild, T.bbox_bits,
+                 T.hmax_bits, T.box32};
+  P.G = PairGrid{g->cell_face_off, g->face_plane, g->face32, g->site, g->rad, g->rin};
+  MAP_TRY(ensure_t(ctx, ctx->ws_pairs[0], nc + 1, &P.count));
+  const int64_t npool = nc / 32 + (2 * nc < 4096 ? 2 * nc : 4096);
+  int32_t* buf;
+  MAP_TRY(ensure_t(ctx, ctx->ws_pairs[8], (size_t)(nc + npool) * (PAIR_ROW + 1), &buf));
+  MAP_TRY(ensure_t(ctx, ctx->ws_pairs[9], nc, &P.Q.again));
+  P.Q.rows = buf;
+  P.Q.pool = buf + nc * PAIR_ROW;
+  P.Q.first = P.Q.pool + npool * PAIR_ROW;
+  P.Q.next = P.Q.first + nc;
+  P.Q.npool = (int32_t)npool;
+  P.Q.used = ctx->d_counters + 5;
+  P.Q.n_again = ctx->d_counters + 6;
+  CUDA_TRY(cudaMemsetAsync(P.Q.used, 0, 2 * sizeof(unsigned long long), s));
+  CUDA_TRY(cudaMemsetAsync(P.count + nc, 0, sizeof(int64_t), s));
   // many particles per cell (few, large cells): one warp per cell
-  const bool per_warp = T.n > 16 * nc;
-  if (per_warp)
-    pair_walk_warp<false><<<(unsigned)((nc + 3) / 4), tpb, 0, s>>>(nc, nullptr, PT, PG, count, nullptr, rows, nullptr);
+  P.per_warp = T.n > 16 * nc;
+  if (P.per_warp) {
+    pair_walk_warp<false><<<nblk(nc, 4), tpb, 0, s>>>(nc, P.T, P.G, P.count, P.Q, nullptr, nullptr, 0); ++ctx->launches;
+    CUDA_TRY(cudaGetLastError());
+    mark_again<<<nblk(nc, 256), 256, 0, s>>>(nc, P.count, P.Q); ++ctx->launches;
+  } else {
+    const unsigned blocks = nblk(nc, PT_WARPS * 32);
+    pair_traverse<WALK_ROWS><<<blocks, PT_WARPS * 32, 0, s>>>(nc, P.order, P.T, P.G, P.count, P.Q, nullptr, nullptr, 0);
+    ++ctx->launches;
+    CUDA_TRY(cudaGetLastError());
+    row_filter<<<nblk(nc, 4), 128, 0, s>>>(nc, P.order, P.T, P.G, P.Q, P.count); ++ctx->launches;
+    CUDA_TRY(cudaGetLastError());
+    pair_traverse<WALK_COUNT><<<blocks, PT_WARPS * 32, 0, s>>>(nc, P.order, P.T, P.G, P.count, P.Q, nullptr, nullptr, 0);
+    ++ctx->launches;
+  }
+  CUDA_TRY(cudaGetLastError());
+  return MAP_OK;
+}
+
+// The rows and the cells walked again into the list (nothing is written when
+// off[nc] exceeds cap).
+int walk_list(map_ctx* ctx, const PairWalk& P, int64_t nc, const int64_t* off, int32_t* list, int64_t cap,
+              cudaStream_t s) {
+  place_rows<<<nblk(nc * 32, 128), 128, 0, s>>>(nc, P.count, off, P.Q, list, cap); ++ctx->launches;
+  CUDA_TRY(cudaGetLastError());
+  if (P.per_warp)
+    pair_walk_warp<true><<<nblk(nc, 4), 128, 0, s>>>(nc, P.T, P.G, nullptr, P.Q, off, list, cap);
   else
-    pair_traverse<false><<<nblk(nc, PT_WARPS * 32), PT_WARPS * 32, 0, s>>>(nc, order, PT, PG, count, nullptr, rows, nullptr);
+    pair_traverse<WALK_FILL><<<nblk(nc, PT_WARPS * 32), PT_WARPS * 32, 0, s>>>(nc, P.order, P.T, P.G, nullptr, P.Q, off,
+                                                                               list, cap);
   ++ctx->launches;
   CUDA_TRY(cudaGetLastError());
-  tb = 0;
+  return MAP_OK;
+}
+
+}  // namespace
+
+int pairs_build(map_ctx* ctx, const PreparedGrid* g, cudaStream_t s, const PairBufs& out) {
+  const int64_t nc = g->ncell;
+  PairWalk P;
+  MAP_TRY(walk_rows(ctx, g, s, P));
+  int64_t* count = P.count;
+  int64_t* off;
+  MAP_TRY(ensure_t(ctx, out.off ? *out.off : ctx->ws_pairs[1], nc + 1, &off));
+  size_t tb = 0;
   CUDA_TRY(cub::DeviceScan::ExclusiveSum(nullptr, tb, count, off, nc + 1, s));
   MAP_TRY(ctx_ensure(ctx, ctx->cub_tmp, tb));
   CUDA_TRY(cub::DeviceScan::ExclusiveSum(ctx->cub_tmp.p, tb, count, off, nc + 1, s));
@@ -476,19 +797,7 @@ int pairs_build(map_ctx* ctx, const PreparedGrid* g, cudaStream_t s, const PairB
   // map_copy_pairs sort each cell's entries by particle index when read
   int32_t* list;
   MAP_TRY(ensure_t(ctx, out.idx ? *out.idx : ctx->ws_pairs[3], np + 1, &list));
-  // rows that fit go straight to the list; the other cells are walked again
-  int32_t* ovf;
-  MAP_TRY(ensure_t(ctx, ctx->ws_pairs[9], nc, &ovf));
-  unsigned long long* d_novf = ctx->d_counters + 6;
-  CUDA_TRY(cudaMemsetAsync(d_novf, 0, sizeof(unsigned long long), s));
-  place_rows<<<nblk(nc * 32, tpb), tpb, 0, s>>>(nc, count, off, rows, list, ovf, d_novf); ++ctx->launches;
-  CUDA_TRY(cudaGetLastError());
-  if (per_warp)
-    pair_walk_warp<true><<<(unsigned)((nc + 3) / 4), tpb, 0, s>>>(nc, ovf, PT, PG, nullptr, off, list, d_novf);
-  else
-    pair_traverse<true><<<nblk(nc, PT_WARPS * 32), PT_WARPS * 32, 0, s>>>(nc, ovf, PT, PG, nullptr, off, list, d_novf);
-  ++ctx->launches;
-  CUDA_TRY(cudaGetLastError());
+  MAP_TRY(walk_list(ctx, P, nc, off, list, INT64_MAX, s));
   ctx->n_pairs = np;
   ctx->pair_off = off;
   ctx->pair_idx = list;
@@ -537,56 +846,19 @@ int items_build(map_ctx* ctx, const int64_t* off, int64_t nc, int64_t np, int ta
 int pairs_build_graph(map_ctx* ctx, const PreparedGrid* g, cudaStream_t s, const PairBufs& out, int64_t cap_pairs,
                       int64_t cap_items) {
   if (!out.off || !out.idx || !out.items || !out.ioff || !out.part) return MAP_EINVAL;
-  DevTree& T = ctx->tree;
   const int64_t nc = g->ncell;
-  const int tpb = 128;
-  uint64_t *k_in, *k_out;
-  int32_t *o_in, *order;
-  MAP_TRY(ensure_t(ctx, ctx->ws_pairs[4], nc, &k_in));
-  MAP_TRY(ensure_t(ctx, ctx->ws_pairs[5], nc, &k_out));
-  MAP_TRY(ensure_t(ctx, ctx->ws_pairs[6], nc, &o_in));
-  MAP_TRY(ensure_t(ctx, ctx->ws_pairs[14], nc, &order));
-  site_keys<<<nblk(nc, 256), 256, 0, s>>>(nc, g->site, k_in, o_in); ++ctx->launches;
-  CUDA_TRY(cudaGetLastError());
-  size_t tb = 0;
-  CUDA_TRY(cub::DeviceRadixSort::SortPairs(nullptr, tb, k_in, k_out, o_in, order, nc, 0, 30, s));
-  MAP_TRY(ctx_ensure(ctx, ctx->cub_tmp, tb));
-  CUDA_TRY(cub::DeviceRadixSort::SortPairs(ctx->cub_tmp.p, tb, k_in, k_out, o_in, order, nc, 0, 30, s));
-  PairTree PT{T.xs, T.ys, T.zs, T.hs, T.hs32, T.split, T.idx, T.begin, T.end, T.first_child, T.nchild, T.bbox_bits,
-              T.hmax_bits, T.box32};
-  PairGrid PG{g->cell_face_off, g->face_plane, g->face32, g->site, g->rad, g->rin};
-  int64_t *count, *off;
-  MAP_TRY(ensure_t(ctx, ctx->ws_pairs[0], nc + 1, &count));
+  PairWalk P;
+  MAP_TRY(walk_rows(ctx, g, s, P));
+  int64_t* count = P.count;
+  int64_t* off;
   MAP_TRY(ensure_t(ctx, *out.off, nc + 1, &off));
-  int32_t* rows;
-  MAP_TRY(ensure_t(ctx, ctx->ws_pairs[8], (size_t)nc * PAIR_ROW, &rows));
-  CUDA_TRY(cudaMemsetAsync(count + nc, 0, sizeof(int64_t), s));
-  const bool per_warp = T.n > 16 * nc;
-  if (per_warp)
-    pair_walk_warp<false><<<(unsigned)((nc + 3) / 4), tpb, 0, s>>>(nc, nullptr, PT, PG, count, nullptr, rows, nullptr);
-  else
-    pair_traverse<false><<<nblk(nc, PT_WARPS * 32), PT_WARPS * 32, 0, s>>>(nc, order, PT, PG, count, nullptr, rows, nullptr);
-  ++ctx->launches;
-  CUDA_TRY(cudaGetLastError());
-  tb = 0;
+  size_t tb = 0;
   CUDA_TRY(cub::DeviceScan::ExclusiveSum(nullptr, tb, count, off, nc + 1, s));
   MAP_TRY(ctx_ensure(ctx, ctx->cub_tmp, tb));
   CUDA_TRY(cub::DeviceScan::ExclusiveSum(ctx->cub_tmp.p, tb, count, off, nc + 1, s));
   int32_t* list;
   MAP_TRY(ensure_t(ctx, *out.idx, cap_pairs + 1, &list));
-  int32_t* ovf;
-  MAP_TRY(ensure_t(ctx, ctx->ws_pairs[9], nc, &ovf));
-  unsigned long long* d_novf = ctx->d_counters + 6;
-  CUDA_TRY(cudaMemsetAsync(d_novf, 0, sizeof(unsigned long long), s));
-  place_rows<<<nblk(nc * 32, tpb), tpb, 0, s>>>(nc, count, off, rows, list, ovf, d_novf, cap_pairs); ++ctx->launches;
-  CUDA_TRY(cudaGetLastError());
-  if (per_warp)
-    pair_walk_warp<true><<<(unsigned)((nc + 3) / 4), tpb, 0, s>>>(nc, ovf, PT, PG, nullptr, off, list, d_novf,
-                                                                  cap_pairs);
-  else
-    pair_traverse<true><<<nblk(nc, PT_WARPS * 32), PT_WARPS * 32, 0, s>>>(nc, ovf, PT, PG, nullptr, off, list, d_novf, cap_pairs);
-  ++ctx->launches;
-  CUDA_TRY(cudaGetLastError());
+  MAP_TRY(walk_list(ctx, P, nc, off, list, cap_pairs, s));
   // the work items (the item size from the device-side pair count)
   const int64_t tgt = (int64_t)ctx->item_target * ctx->sm_count * 24;
   int64_t *icnt, *ioff;
