@@ -23,13 +23,24 @@
 // bisection rules are those of the per-particle definition; only the order
 // of the sums differs.
 //
-// Mixed build: Newton and bisection sums in FP32 (on hi/lo-split
-// coordinates); the Newton iterate, its step and the list-coverage tests in
-// FP32 too (hfact as an FP32 hi/lo pair), the converged step applied in FP64;
-// stop at |dh| < 1e-6 h.  FP64 build: every sum in FP64 behind an FP32
-// distance screen with a 1e-5 relative margin, stop at 1e-10.
-#include <type_traits>
-
+// What bounds it is latency: one warp's chain of gathers, per particle about
+// 3.5 sums of some 100 terms each.  So a pass keeps HS_MLP candidates per
+// lane in flight, and a particle's own candidates are held in registers as
+// offsets from it (they do not depend on h), so that its later Newton steps
+// load nothing.  Where the leaf's list is longer than its buffer, each lane
+// keeps the candidates it found within reach of the particle and its later
+// steps add those alone, in the order a full pass adds them.
+//
+// Both builds solve in FP32: Newton and bisection sums on hi/lo-split
+// coordinates, the iterate, its step and the list-coverage tests in FP32
+// (hfact as an FP32 hi/lo pair), the converged step (|dh| < 1e-6 h) applied in
+// FP64.  That is the mixed build's h, 5e-8 from the root.  The FP64 build then
+// takes one FP64 step of third order from there: with S(h) = sum_b w(r_ab/h),
+// Eq. (7) is S(h) = pi hfact^3, and Halley's step from the FP64 sums of w,
+// q w' and q^2 w'' + 2 q w' leaves an error of (5e-8)^3.  FP64 sums at every
+// Newton step (4.2 per particle on a pipe at about 1/74 of the FP32 rate, to
+// |dh| < 1e-10 h) took 77 ms at 2^20 clumpy particles; now 22 ms, of which the
+// FP32 solve is 11 ms (mixed: 12.9 ms before; 60,000 particles 5.2 -> 2.0 ms).
 #include "internal.cuh"
 
 namespace {
@@ -42,6 +53,11 @@ constexpr int HS_CAP = 1024;    // candidate positions held per warp (a multiple
 // most its 8 children, so at most 8 + 7 * 21 = 155 entries are live.
 constexpr int HS_STK = 160;
 constexpr int HS_PCAP = 512;   // one particle's own candidates (within 2.5 h of it)
+constexpr int HS_WIN = 8;      // sorted positions per warp, which takes the leaves that start among them: about
+                               // one leaf (7 particles on average), so that a snapshot of 60,000 gives 7,500
+                               // warps (32 positions: 1,875, one wave as long as its slowest four leaves)
+constexpr int HS_MLP = 2;      // candidates per lane in flight during a pass (4: more registers, 12.6 ms at 2^20)
+constexpr int HS_REG = 6;      // own candidates per lane held in registers (192 per particle; 113 on average)
 constexpr unsigned FULL = 0xffffffffu;
 
 struct HsTree {
@@ -59,31 +75,27 @@ struct HsWarp {
   int32_t stk[HS_STK];
 };
 
-// Candidate list held by one warp (values uniform across its lanes); S is
-// the build's type for h (FP32 in the mixed build, FP64 in the FP64 build).
-template <typename S>
+// Candidate list held by one warp (values uniform across its lanes).
 struct HsBuf {
   float q[6];       // query box: the leaf's outward-rounded FP32 box
-  S R;              // gather radius
+  float R;          // gather radius
   int nr;           // ranges held
   bool rng_done;    // the walk finished: the ranges cover every candidate
   int64_t total;    // positions in the ranges held
   bool expanded;    // cand holds all of them
   int64_t pk;       // the particle whose own list pcand holds (-1: none)
-  S pR;             // its radius
+  float pR;         // its radius
   int pn;           // its length
+  float cR;         // radius of the lanes' own finds of a long list (pcand[32 i + lane]); < 0: none
 };
 
-__device__ __forceinline__ double w_m4(double q) {
-  if (q < 1.0) return 1.0 - 1.5 * q * q + 0.75 * q * q * q;
-  if (q < 2.0) { const double t = 2.0 - q; return 0.25 * t * t * t; }
-  return 0.0;
-}
-__device__ __forceinline__ double dw_m4(double q) {
-  if (q < 1.0) return -3.0 * q + 2.25 * q * q;
-  if (q < 2.0) { const double t = 2.0 - q; return -0.75 * t * t; }
-  return 0.0;
-}
+// The current particle's candidates in registers, as offsets from it: lane
+// l's entries are the positions l, l + 32, ... of its own list, or the lane's
+// finds of a long list, in the order the lists are summed.
+struct HsOwn {
+  float x[HS_REG], y[HS_REG], z[HS_REG];
+  int n;  // this lane's entries
+};
 
 // True when no point of box b is within R of box q.  Both boxes are rounded
 // outward; the FP32 arithmetic on coordinates in the unit cube is covered by
@@ -114,14 +126,12 @@ struct HsWalk {
   unsigned m;     // pending range children (leaves, or nodes taken whole)
 };
 
-__device__ __forceinline__ float walk_margin(double R) { return (float)(R + 1e-6) * 1.000001f; }
 __device__ __forceinline__ float walk_margin(float R) { return (R + 1e-6f) * 1.000001f; }
 
-template <typename S>
-__device__ __forceinline__ void walk_begin(const HsTree& T, HsWarp& W, HsWalk& it, S R, int& nr) {
+__device__ __forceinline__ void walk_begin(const HsTree& T, HsWarp& W, HsWalk& it, float R, int& nr) {
   __syncwarp();
   it.Rm = walk_margin(R);
-  it.Rin = (float)R;
+  it.Rin = R;
   it.m = 0u;
   it.c0 = 0;
   it.sp = 0;
@@ -192,86 +202,127 @@ __device__ int walk_next(const HsTree& T, HsWarp& W, HsWalk& it, const float* q,
   return nr;
 }
 
-// Lane partial sums of w(q) and 3 w + q w'(q) over list[0, cnt) for the
-// particle at sorted position k.  A lane takes positions lane, lane + 32, ...
-// in that order; two of them per pass, with the loads of both issued before
-// either term is added (the order of the additions is unchanged).  With keep
-// set, the candidates with q^2 < keep_q2 are also appended, in list order, to
-// keep[*nkeep ...] (*nkeep = -1 when they do not fit in HS_PCAP).
-template <bool F32, typename S>
-__device__ __forceinline__ void warp_accum(const HsTree& T, const int32_t* list, int cnt, int64_t k, S h,
-                                           float& s32, float& d32, double& s64, double& d64, int32_t* keep,
-                                           float keep_q2, int* nkeep) {
-  const int lane = threadIdx.x & 31;
-  const unsigned lt = (1u << lane) - 1u;
-  const float* P0 = T.split + 6 * k;
-  const float hx = P0[0], lx = P0[1], hy = P0[2], ly = P0[3], hz = P0[4], lz = P0[5];
-  const float inv_hf = 1.0f / (float)h;
-  double x = 0.0, y = 0.0, z = 0.0, R2 = 0.0, inv_h = 0.0;
-  if (!F32) {
-    x = T.xs[k]; y = T.ys[k]; z = T.zs[k];
-    R2 = 4.0 * (double)h * (double)h;
-    inv_h = 1.0 / (double)h;
+// The particle at sorted position k, FP32 hi/lo.
+struct HsPoint {
+  float hx, lx, hy, ly, hz, lz;
+};
+__device__ __forceinline__ HsPoint point_of(const HsTree& T, int64_t k) {
+  const float2* P = reinterpret_cast<const float2*>(T.split + 6 * k);
+  const float2 a = __ldg(P), b = __ldg(P + 1), c = __ldg(P + 2);
+  return HsPoint{a.x, a.y, b.x, b.y, c.x, c.y};
+}
+
+// One candidate at the offset (ox, oy, oz): w(q) and 3 w + q w'(q) added when
+// inside; returns q^2.  The sums' roundings are written out, so that h does not
+// move with the compiler's choice of what to fuse: q^2 in the order x^2, y^2,
+// z^2 for bisection and y^2, x^2, z^2 for Newton, which also needs d.
+template <bool NEWTON>
+__device__ __forceinline__ float add_term(float ox, float oy, float oz, float inv_h, float& s, float& d) {
+  const float dx = ox * inv_h, dy = oy * inv_h, dz = oz * inv_h;
+  const float q2 = NEWTON ? __fmaf_rn(dz, dz, __fmaf_rn(dx, dx, __fmul_rn(dy, dy)))
+                          : __fmaf_rn(dz, dz, __fmaf_rn(dy, dy, __fmul_rn(dx, dx)));
+  if (q2 >= 4.f) return q2;
+  const float q = sqrtf(q2);
+  float w, dwq;
+  if (q < 1.f) {
+    w = __fmaf_rn(__fmul_rn(0.75f, q2), q, __fmaf_rn(-1.5f, q2, 1.f));
+    dwq = -3.f * q2 + 2.25f * q2 * q;
+  } else {
+    const float t = 2.f - q;
+    w = __fmul_rn(__fmul_rn(__fmul_rn(0.25f, t), t), t);
+    dwq = -0.75f * t * t * q;
   }
-  // q^2 of one candidate (FP32, as the screen), its terms added when inside
-  auto term = [&](int64_t c, float2 a, float2 b, float2 cc) -> float {
-    const float dx = ((a.x - hx) + (a.y - lx)) * inv_hf;
-    const float dy = ((b.x - hy) + (b.y - ly)) * inv_hf;
-    const float dz = ((cc.x - hz) + (cc.y - lz)) * inv_hf;
-    const float q2 = dx * dx + dy * dy + dz * dz;
-    if (F32) {
-      if (q2 >= 4.f) return q2;
-      const float q = sqrtf(q2);
-      float w, dwq;
-      if (q < 1.f) { w = 1.f - 1.5f * q2 + 0.75f * q2 * q; dwq = -3.f * q2 + 2.25f * q2 * q; }
-      else { const float t = 2.f - q; w = 0.25f * t * t * t; dwq = -0.75f * t * t * q; }
-      s32 += w;
-      d32 += 3.f * w + dwq;
-    } else {
-      if (q2 > 4.00004f) return q2;  // FP32 screen, 1e-5 relative margin
-      const double ex = T.xs[c] - x, ey = T.ys[c] - y, ez = T.zs[c] - z;
-      const double r2 = ex * ex + ey * ey + ez * ez;
-      if (r2 >= R2) return q2;
-      const double q = sqrt(r2) * inv_h;
-      const double w = w_m4(q);
-      s64 += w;
-      d64 += 3.0 * w + q * dw_m4(q);
+  s = __fadd_rn(s, w);
+  if (NEWTON) d = __fadd_rn(d, 3.f * w + dwq);
+  return q2;
+}
+
+// f(position, offset x, y, z, valid) for list[0, cnt): a lane takes positions
+// lane, lane + 32, ... in that order, HS_MLP of them per round with their
+// loads issued together; every lane calls f, for all of a round's positions.
+template <typename F>
+__device__ __forceinline__ void for_list(const HsTree& T, const int32_t* list, int cnt, const HsPoint& p, F f) {
+  const int lane = threadIdx.x & 31;
+  for (int j0 = 0; j0 < cnt; j0 += 32 * HS_MLP) {
+    int32_t c[HS_MLP];
+    float2 a[HS_MLP], b[HS_MLP], e[HS_MLP];
+#pragma unroll
+    for (int u = 0; u < HS_MLP; ++u) {
+      const int j = j0 + 32 * u + lane;
+      c[u] = list[j < cnt ? j : cnt - 1];
+      const float2* P = reinterpret_cast<const float2*>(T.split + 6 * (int64_t)c[u]);
+      a[u] = __ldg(P); b[u] = __ldg(P + 1); e[u] = __ldg(P + 2);
     }
-    return q2;
-  };
-  auto append = [&](bool pred, int32_t v) {
-    const unsigned m = __ballot_sync(FULL, pred);
-    if (*nkeep < 0) return;
-    if (*nkeep + __popc(m) > HS_PCAP) { *nkeep = -1; return; }
-    if (pred) keep[*nkeep + __popc(m & lt)] = v;
-    *nkeep += __popc(m);
-  };
-  for (int j0 = 0; j0 < cnt; j0 += 64) {
-    const int j = j0 + lane, j1 = j + 32;
-    const bool v0 = j < cnt, v1 = j1 < cnt;
-    int32_t c0 = 0, c1 = 0;
-    float2 a = make_float2(0.f, 0.f), b = a, c = a, a1 = a, b1 = a, cc1 = a;
-    if (v0) {
-      c0 = list[j];
-      const float2* P = reinterpret_cast<const float2*>(T.split + 6 * (int64_t)c0);
-      a = P[0]; b = P[1]; c = P[2];
-    }
-    if (v1) {
-      c1 = list[j1];
-      const float2* Q = reinterpret_cast<const float2*>(T.split + 6 * (int64_t)c1);
-      a1 = Q[0]; b1 = Q[1]; cc1 = Q[2];
-    }
-    const float q0 = v0 ? term(c0, a, b, c) : 1e30f;
-    const float q1 = v1 ? term(c1, a1, b1, cc1) : 1e30f;
-    if (keep) {
-      append(v0 && q0 < keep_q2, c0);
-      append(v1 && q1 < keep_q2, c1);
+#pragma unroll
+    for (int u = 0; u < HS_MLP; ++u) {
+      if (j0 + 32 * u >= cnt) break;
+      f(c[u], (a[u].x - p.hx) + (a[u].y - p.lx), (b[u].x - p.hy) + (b[u].y - p.ly),
+        (e[u].x - p.hz) + (e[u].y - p.lz), j0 + 32 * u + lane < cnt);
     }
   }
 }
 
-__device__ __forceinline__ float rcbrt_s(float v) { return rcbrtf(v); }
-__device__ __forceinline__ double rcbrt_s(double v) { return rcbrt(v); }
+// Lane partial sums of w(q) and 3 w + q w'(q) over list[0, cnt).
+template <bool NEWTON>
+__device__ __forceinline__ void warp_accum(const HsTree& T, const int32_t* list, int cnt, const HsPoint& p, float inv_h,
+                                           float& s, float& d) {
+  for_list(T, list, cnt, p, [&](int32_t, float ox, float oy, float oz, bool on) {
+    if (on) add_term<NEWTON>(ox, oy, oz, inv_h, s, d);
+  });
+}
+
+// The same, and the candidates with q^2 < keep_q2 are appended, in list
+// order, to keep[0, *nkeep) (*nkeep = -1 when they do not fit in HS_PCAP).
+template <bool NEWTON>
+__device__ __forceinline__ void warp_accum_keep(const HsTree& T, const int32_t* list, int cnt, const HsPoint& p,
+                                                float inv_h, float& s, float& d, int32_t* keep, float keep_q2,
+                                                int* nkeep) {
+  const unsigned lt = (1u << (threadIdx.x & 31)) - 1u;
+  int nk = 0;
+  for_list(T, list, cnt, p, [&](int32_t c, float ox, float oy, float oz, bool on) {
+    const float q2 = on ? add_term<NEWTON>(ox, oy, oz, inv_h, s, d) : 1e30f;
+    const unsigned m = __ballot_sync(FULL, on && q2 < keep_q2);
+    if (nk < 0) return;
+    if (nk + __popc(m) > HS_PCAP) { nk = -1; return; }
+    if (on && q2 < keep_q2) keep[nk + __popc(m & lt)] = c;
+    nk += __popc(m);
+  });
+  *nkeep = nk;
+}
+
+// The same over one chunk of a long list; a lane's candidates with q^2 <
+// keep_q2 are appended to its own column keep[32 i + lane], i < HS_PCAP / 32
+// (nl counts past that when they do not fit).
+template <bool NEWTON>
+__device__ __forceinline__ void warp_accum_lane(const HsTree& T, const int32_t* list, int cnt, const HsPoint& p,
+                                                float inv_h, float& s, float& d, int32_t* keep, float keep_q2,
+                                                int& nl) {
+  const int lane = threadIdx.x & 31;
+  for_list(T, list, cnt, p, [&](int32_t c, float ox, float oy, float oz, bool on) {
+    if (!on) return;
+    const float q2 = add_term<NEWTON>(ox, oy, oz, inv_h, s, d);
+    if (q2 < keep_q2) {
+      if (keep && nl < HS_PCAP / 32) keep[32 * nl + lane] = c;
+      ++nl;
+    }
+  });
+}
+
+// The offsets of this lane's n entries col[0], col[32], ... into registers.
+__device__ __forceinline__ void own_load(const HsTree& T, const int32_t* col, int n, const HsPoint& p, HsOwn& O) {
+  O.n = n;
+#pragma unroll
+  for (int i = 0; i < HS_REG; ++i) {
+    O.x[i] = O.y[i] = O.z[i] = 0.f;
+    if (i < n) {
+      const float2* P = reinterpret_cast<const float2*>(T.split + 6 * (int64_t)col[32 * i]);
+      const float2 a = __ldg(P), b = __ldg(P + 1), c = __ldg(P + 2);
+      O.x[i] = (a.x - p.hx) + (a.y - p.lx);
+      O.y[i] = (b.x - p.hy) + (b.y - p.ly);
+      O.z[i] = (c.x - p.hz) + (c.y - p.lz);
+    }
+  }
+}
 
 template <typename V>
 __device__ __forceinline__ V warp_total(V v) {
@@ -299,11 +350,11 @@ __device__ int expand(HsWarp& W, int nr, int& r, int& off) {
 }
 
 // Gathers the candidate ranges for radius R, and their positions when they fit.
-template <typename S>
-__device__ __forceinline__ void regather(const HsTree& T, HsWarp& W, HsBuf<S>& B, S R) {
+__device__ __forceinline__ void regather(const HsTree& T, HsWarp& W, HsBuf& B, float R) {
   const int lane = threadIdx.x & 31;
   HsWalk it;
   B.R = R;
+  B.cR = -1.f;
   walk_begin(T, W, it, R, B.nr);
   B.nr = walk_next(T, W, it, B.q, B.nr);
   B.rng_done = walk_done(it);
@@ -319,95 +370,189 @@ __device__ __forceinline__ void regather(const HsTree& T, HsWarp& W, HsBuf<S>& B
   }
 }
 
-// n(h) and dn/dh for the particle at sorted position k (warp-uniform result),
-// in the build's type S for h (every test on h and the radii in S).
-template <bool F32, typename S>
-__device__ void warp_density(const HsTree& T, HsWarp& W, HsBuf<S>& B, int64_t k, S h, S& n, S& dn) {
-  float s32 = 0.f, d32 = 0.f;
-  double s64 = 0.0, d64 = 0.0;
-  int none = 0;
-  const bool own = B.pk == k && S(2) * h <= S(0.999) * B.pR && B.pR <= S(8) * h;
-  if (own) {
-    // the particle's own list covers its support at this h
-    warp_accum<F32>(T, W.pcand, B.pn, k, h, s32, d32, s64, d64, nullptr, 0.f, &none);
-  } else {
-    if (S(2) * h > B.R || B.R > S(8) * h) regather(T, W, B, S(2.5) * h);
+// f(list, count) for every chunk of a list that does not fit the position
+// buffer, in the same chunks every time.
+template <typename F>
+__device__ __forceinline__ void for_chunks(const HsTree& T, HsWarp& W, HsBuf& B, F f) {
+  if (B.rng_done) {
+    // the ranges are complete but longer than the position buffer
+    int r = 0, off = 0;
+    while (r < B.nr) {
+      const int c = expand(W, B.nr, r, off);
+      f(W.cand, c);
+    }
+    return;
   }
-  if (own) {
-    // done above
+  // more ranges than their buffer: one resumable walk, range chunk by chunk
+  HsWalk it;
+  int nr;
+  walk_begin(T, W, it, B.R, nr);
+  for (;;) {
+    nr = walk_next(T, W, it, B.q, nr);
+    int r = 0, off = 0;
+    while (r < nr) {
+      const int c = expand(W, nr, r, off);
+      f(W.cand, c);
+    }
+    if (walk_done(it)) break;
+    nr = 0;
+  }
+  B.nr = 0;
+  B.R = -1.f;  // the buffer no longer holds the first ranges: regather next time
+}
+
+// n(h) and dn/dh for the particle at sorted position k (warp-uniform result).
+template <bool NEWTON>
+__device__ __forceinline__ void warp_density(const HsTree& T, HsWarp& W, HsBuf& B, HsOwn& O, int64_t k,
+                                             const HsPoint& p, float h, float& n, float& dn) {
+  const int lane = threadIdx.x & 31;
+  float s = 0.f, d = 0.f;
+  const float inv_h = 1.0f / h;
+  bool held = B.pk == k && 2.f * h <= 0.999f * B.pR && B.pR <= 8.f * h;
+  const bool own = held;
+  bool wide = own && B.pn > 32 * HS_REG;  // its own list, not held in registers
+  if (!own) {
+    if (2.f * h > B.R || B.R > 8.f * h) regather(T, W, B, 2.5f * h);
+    // the lanes' finds of a long list cover its support at this h
+    held = !B.expanded && 2.f * h <= 0.999f * B.cR;
+  }
+  if (held && !wide) {
+#pragma unroll
+    for (int i = 0; i < HS_REG; ++i)
+      if (i < O.n) add_term<NEWTON>(O.x[i], O.y[i], O.z[i], inv_h, s, d);
+    if (!own && __any_sync(FULL, O.n > HS_REG)) {
+      for (int i = HS_REG; i < O.n; ++i) {
+        const HsPoint c = point_of(T, W.pcand[32 * i + lane]);
+        add_term<NEWTON>((c.hx - p.hx) + (c.lx - p.lx), (c.hy - p.hy) + (c.ly - p.ly), (c.hz - p.hz) + (c.lz - p.lz), inv_h, s,
+                 d);
+      }
+      __syncwarp();
+    }
+  } else if (wide) {
+    warp_accum<NEWTON>(T, W.pcand, B.pn, p, inv_h, s, d);
   } else if (B.expanded) {
     // the leaf's list; the first pass for a particle also keeps its own
     // candidates within pR = min(2.5 h, R) of it for the next steps (the
     // leaf's list holds every candidate within R of the leaf's box, so of
     // the particle)
     if (B.pk != k) {
-      const S pR = S(2.5) * h < B.R ? S(2.5) * h : B.R;
-      const float kq = (float)(pR / h);
+      const float pR = 2.5f * h < B.R ? 2.5f * h : B.R;
+      const float kq = pR / h;
       int nk = 0;
-      warp_accum<F32>(T, W.cand, (int)B.total, k, h, s32, d32, s64, d64, W.pcand, kq * kq * 1.00001f, &nk);
+      warp_accum_keep<NEWTON>(T, W.cand, (int)B.total, p, inv_h, s, d, W.pcand, kq * kq * 1.00001f, &nk);
       __syncwarp();
       B.pk = k;
-      B.pR = nk >= 0 ? pR : S(0);  // 0: nothing kept (it did not fit)
+      B.pR = nk >= 0 ? pR : 0.f;  // 0: nothing kept (it did not fit)
       B.pn = nk >= 0 ? nk : 0;
+      if (nk <= 32 * HS_REG) own_load(T, W.pcand + lane, (B.pn - lane + 31) >> 5, p, O);
     } else {
-      warp_accum<F32>(T, W.cand, (int)B.total, k, h, s32, d32, s64, d64, nullptr, 0.f, &none);
-    }
-  } else if (B.rng_done) {
-    // the ranges are complete but longer than the position buffer
-    int r = 0, off = 0;
-    while (r < B.nr) {
-      const int c = expand(W, B.nr, r, off);
-      warp_accum<F32>(T, W.cand, c, k, h, s32, d32, s64, d64, nullptr, 0.f, &none);
+      warp_accum<NEWTON>(T, W.cand, (int)B.total, p, inv_h, s, d);
     }
   } else {
-    // more ranges than their buffer: one resumable walk, range chunk by chunk
-    HsWalk it;
-    int nr;
-    walk_begin(T, W, it, B.R, nr);
-    for (;;) {
-      nr = walk_next(T, W, it, B.q, nr);
-      int r = 0, off = 0;
-      while (r < nr) {
-        const int c = expand(W, nr, r, off);
-        warp_accum<F32>(T, W.cand, c, k, h, s32, d32, s64, d64, nullptr, 0.f, &none);
+    // a long list: the particle's own list keeps pcand when there is one
+    const bool room = B.pk != k;
+    const float cR = 2.5f * h < B.R ? 2.5f * h : B.R;
+    const float kq = cR / h;
+    int nl = 0;
+    for_chunks(T, W, B, [&](const int32_t* list, int c) {
+      warp_accum_lane<NEWTON>(T, list, c, p, inv_h, s, d, room ? W.pcand : nullptr, kq * kq * 1.00001f, nl);
+    });
+    __syncwarp();
+    B.cR = -1.f;
+    if (room && B.R > 0.f && !__any_sync(FULL, nl > HS_PCAP / 32)) {
+      B.cR = cR;
+      own_load(T, W.pcand + lane, nl, p, O);
+    }
+  }
+  const float norm = inv_h * inv_h * inv_h * (float)(1.0 / MAP_PI);
+  n = warp_total(s) * norm;
+  dn = -warp_total(d) * norm * inv_h;
+}
+
+// FP64 sums of w(q), q w'(q) and q^2 w''(q) + 2 q w'(q) at h over list[0,
+// cnt) around the particle at sorted position k: the candidates an FP32
+// distance screen (1e-5 relative margin) leaves are packed into buf (at least
+// 64 entries), so that the FP64 terms run with full warps.
+__device__ __forceinline__ void accum64(const HsTree& T, const int32_t* list, int cnt, const HsPoint& p, int64_t k,
+                                        double h, int32_t* buf, double& s, double& d, double& e) {
+  const int lane = threadIdx.x & 31;
+  const unsigned lt = (1u << lane) - 1u;
+  const double x = T.xs[k], y = T.ys[k], z = T.zs[k], inv_h = 1.0 / h;
+  const float ih = (float)inv_h;
+  int nb = 0;
+  auto drain = [&](int m) {  // the first m (<= 32) of buf
+    __syncwarp();
+    if (lane < m) {
+      const int64_t c = buf[lane];
+      const double ex = (T.xs[c] - x) * inv_h, ey = (T.ys[c] - y) * inv_h, ez = (T.zs[c] - z) * inv_h;
+      const double q2 = ex * ex + ey * ey + ez * ez;
+      const double q = sqrt(q2), q3 = q2 * q;
+      if (q < 1.0) {
+        s += 1.0 - 1.5 * q2 + 0.75 * q3;
+        d += 2.25 * q3 - 3.0 * q2;
+        e += 9.0 * (q3 - q2);
+      } else if (q < 2.0) {
+        const double t = 2.0 - q, t2 = t * t;
+        s += 0.25 * t2 * t;
+        d -= 0.75 * t2 * q;
+        e += 1.5 * t * q * (q - t);
       }
-      if (walk_done(it)) break;
-      nr = 0;
     }
-    B.nr = 0;
-    B.R = S(-1);  // the buffer no longer holds the first ranges: regather next time
-  }
-  if (F32) {
-    const float ih = 1.0f / (float)h;
-    const float norm = ih * ih * ih * (float)(1.0 / MAP_PI);
-    n = (S)(warp_total(s32) * norm);
-    dn = (S)(-warp_total(d32) * norm * ih);
+    __syncwarp();
+  };
+  for_list(T, list, cnt, p, [&](int32_t c, float ox, float oy, float oz, bool on) {
+    const float dx = ox * ih, dy = oy * ih, dz = oz * ih;
+    const bool in = on && dx * dx + dy * dy + dz * dz <= 4.00004f;
+    const unsigned m = __ballot_sync(FULL, in);
+    if (in) buf[nb + __popc(m & lt)] = c;
+    nb += __popc(m);
+    if (nb >= 32) {
+      drain(32);
+      nb -= 32;
+      const int32_t v = lane < nb ? buf[32 + lane] : 0;
+      __syncwarp();
+      if (lane < nb) buf[lane] = v;
+    }
+  });
+  if (nb) drain(nb);
+}
+
+// The FP64 build's sums at h, from the shortest list that covers its support.
+__device__ __forceinline__ void density64(const HsTree& T, HsWarp& W, HsBuf& B, int64_t k, const HsPoint& p, double h,
+                                          double& s, double& d, double& e) {
+  s = d = e = 0.0;
+  const float hf = (float)h;
+  int32_t* buf = W.stk;  // free outside a walk
+  if (B.pk == k && 2.f * hf <= 0.999f * B.pR) {
+    accum64(T, W.pcand, B.pn, p, k, h, buf, s, d, e);
   } else {
-    const double ih = 1.0 / h;
-    const double norm = ih * ih * ih * (1.0 / MAP_PI);
-    n = warp_total(s64) * norm;
-    dn = -warp_total(d64) * norm * ih;
+    if (2.f * hf > 0.999f * B.R) regather(T, W, B, 2.5f * hf);
+    if (B.expanded) accum64(T, W.cand, (int)B.total, p, k, h, buf, s, d, e);
+    else for_chunks(T, W, B, [&](const int32_t* list, int c) {
+      // a walk between chunks uses the stack: the packing buffer is local to a chunk
+      accum64(T, list, c, p, k, h, W.pcand, s, d, e);
+    });
+    if (!B.expanded) { B.pk = -1; B.cR = -1.f; }  // pcand was used
   }
+  s = warp_total(s);
+  d = warp_total(d);
+  e = warp_total(e);
 }
 
 template <bool MIXED>
 __global__ void __launch_bounds__(HS_WARPS * 32)
-    h_solve_leaves(int64_t n, HsTree T, const double* __restrict__ h0s, double hfact, double tol, double* hout,
-                   int32_t* route) {
-  // the build's type for h: the mixed build iterates in FP32 (its sums are
-  // FP32, and GB300's FP64 rate is about 1/74 of its FP32 rate)
-  using S = typename std::conditional<MIXED, float, double>::type;
-  const S hf_s = (S)hfact, hf3_s = (S)(hfact / 3.0), tol_s = (S)tol;
-  const S hf_lo = (S)(hfact - (double)hf_s);
+    h_solve_leaves(int64_t n, HsTree T, const double* __restrict__ h0s, double hfact, double* hout, int32_t* route) {
+  const float hf_s = (float)hfact, hf3_s = (float)(hfact / 3.0), tol_s = 1e-6f;
+  const float hf_lo = (float)(hfact - (double)hf_s);
   __shared__ HsWarp sw[HS_WARPS];
   HsWarp& W = sw[threadIdx.x >> 5];
   const int lane = threadIdx.x & 31;
-  const int64_t k0 = (blockIdx.x * (int64_t)HS_WARPS + (threadIdx.x >> 5)) * 32;
+  const int64_t k0 = (blockIdx.x * (int64_t)HS_WARPS + (threadIdx.x >> 5)) * HS_WIN;
   if (k0 >= n) return;  // whole warp
-  // leaves whose first particle lies in this warp's window of 32 positions
+  // leaves whose first particle lies in this warp's window
   int leaf = -1;
   bool head = false;
-  if (k0 + lane < n) {
+  if (lane < HS_WIN && k0 + lane < n) {
     leaf = T.owner[k0 + lane];
     head = T.nb[leaf] == k0 + lane;
   }
@@ -420,42 +565,47 @@ __global__ void __launch_bounds__(HS_WARPS * 32)
     double gmax = 0.0;
     for (int64_t k = a0 + lane; k < a1; k += 32) gmax = fmax(gmax, h0s[k]);
     for (int o = 16; o > 0; o >>= 1) gmax = fmax(gmax, __shfl_xor_sync(FULL, gmax, o));
-    HsBuf<S> B;
+    HsBuf B;
 #pragma unroll
     for (int i = 0; i < 6; ++i) B.q[i] = T.box32[8 * (int64_t)L + i];
-    B.R = S(-1);
+    B.R = -1.f;
     B.nr = 0;
     B.total = 0;
     B.rng_done = false;
     B.expanded = false;
     B.pk = -1;
-    B.pR = S(0);
+    B.pR = 0.f;
     B.pn = 0;
-    const S R0 = S(2.5) * (S)gmax;
+    B.cR = -1.f;
+    HsOwn O;
+    O.n = 0;
+    const float R0 = 2.5f * (float)gmax;
     for (int64_t k = a0; k < a1; ++k) {
       // the leaf's list for its first particle; later particles keep the
       // list they find while it covers their support (warp_density
       // regathers when 2h > R or R > 8h)
       if (k == a0) regather(T, W, B, R0);
-      // Newton in S: g = h - hfact t, g' = 1 + hfact/3 t^4 dn/dh with t = n^(-1/3)
-      S hs = (S)h0s[k];
-      const S lo_s = hs / S(16), hi_s = hs * S(16);
+      B.cR = -1.f;
+      const HsPoint p = point_of(T, k);
+      // Newton: g = h - hfact t, g' = 1 + hfact/3 t^4 dn/dh with t = n^(-1/3)
+      float hs = (float)h0s[k];
+      const float lo_s = hs / 16.f, hi_s = hs * 16.f;
       double h = 0.0;
       bool ok = false;
       for (int it = 0; it < 30; ++it) {
-        S nn, dn;
-        warp_density<MIXED>(T, W, B, k, hs, nn, dn);
-        const S t = rcbrt_s(nn);
-        S f = hs - hf_s * t;
-        if (MIXED) f -= hf_lo * t;  // hfact as an FP32 pair
-        const S fp = S(1) + hf3_s * (t * t) * (t * t) * dn;
-        const S d = f / fp;
-        const S hn = hs - d;
+        float nn, dn;
+        warp_density<true>(T, W, B, O, k, p, hs, nn, dn);
+        const float t = rcbrtf(nn);
+        float f = hs - hf_s * t;
+        f -= hf_lo * t;  // hfact as an FP32 pair
+        const float fp = 1.f + hf3_s * (t * t) * (t * t) * dn;
+        const float d = f / fp;
+        const float hn = hs - d;
         if (!(hn >= lo_s && hn <= hi_s)) break;
         if ((hn > hs ? hn - hs : hs - hn) < tol_s * hn) {
-          // the mixed build applies its converged step in FP64 (the result
-          // keeps FP64's spacing, not FP32's)
-          h = MIXED ? (double)hs - (double)d : (double)hn;
+          // the converged step is applied in FP64 (the result keeps FP64's
+          // spacing, not FP32's)
+          h = (double)hs - (double)d;
           ok = true;
           break;
         }
@@ -465,12 +615,11 @@ __global__ void __launch_bounds__(HS_WARPS * 32)
       if (!ok) {
         const double g0 = h0s[k];
         const double lo = g0 / 16.0, hi = g0 * 16.0;
-        // (the mixed build bisects on its FP32 sums too: the root moves by
-        // ~1e-7 relative, inside the build's 1e-6, and GB300's FP64 rate
-        // is about 1/74 of its FP32 rate)
+        // bisection on the FP32 sums too: the root moves by ~1e-7 relative,
+        // inside the mixed build's 1e-6 and the FP64 build's last step
         auto g = [&](double hh) {
-          S nn, dn;
-          warp_density<MIXED>(T, W, B, k, (S)hh, nn, dn);
+          float nn, dn;
+          warp_density<false>(T, W, B, O, k, p, (float)hh, nn, dn);
           return hh - hfact * rcbrt((double)nn);
         };
         // Bisection on [lo, hi] needs g(lo) < 0 < g(hi).  g(h)/h is
@@ -507,6 +656,20 @@ __global__ void __launch_bounds__(HS_WARPS * 32)
           }
           h = 0.5 * (a + b);
           r = 1;
+        }
+      }
+      if (!MIXED && r != 2) {
+        // Halley's step on S(h) - pi hfact^3 (S' = -d/h, S'' = e/h^2), again
+        // while a step is so large that its cube shows
+        const double target = MAP_PI * hfact * hfact * hfact;
+        for (int it = 0; it < 30; ++it) {
+          double s, d, e;
+          density64(T, W, B, k, p, h, s, d, e);
+          const double F = s - target;
+          const double u = 2.0 * F * d / (2.0 * d * d - F * e);  // -dh / h times -1: h <- h (1 + u)
+          if (!(fabs(u) < 1e-2)) break;  // S' is 0 (no neighbour inside): the FP32 root stands
+          h += h * u;
+          if (fabs(u) < 2e-6) break;
         }
       }
       if (lane == 0) {
@@ -552,12 +715,12 @@ int h_solve_run(map_ctx* ctx, const double* x, const double* y, const double* z,
   ++ctx->launches;
   CUDA_TRY(cudaGetLastError());
   const HsTree V{T.xs, T.ys, T.zs, T.split, T.begin, T.end, T.first_child, T.nchild, T.owner, T.idx, T.box32};
-  const int64_t warps = (n + 31) / 32;
+  const int64_t warps = (n + HS_WIN - 1) / HS_WIN;
   const unsigned blocks = (unsigned)((warps + HS_WARPS - 1) / HS_WARPS);
   if (ctx->cfg.precision != MAP_FP64)
-    h_solve_leaves<true><<<blocks, HS_WARPS * 32, 0, s>>>(n, V, h0s, ctx->cfg.hfact, 1e-6, h, route);
+    h_solve_leaves<true><<<blocks, HS_WARPS * 32, 0, s>>>(n, V, h0s, ctx->cfg.hfact, h, route);
   else
-    h_solve_leaves<false><<<blocks, HS_WARPS * 32, 0, s>>>(n, V, h0s, ctx->cfg.hfact, 1e-10, h, route);
+    h_solve_leaves<false><<<blocks, HS_WARPS * 32, 0, s>>>(n, V, h0s, ctx->cfg.hfact, h, route);
   ++ctx->launches;
   CUDA_TRY(cudaGetLastError());
   return MAP_OK;
