@@ -16,7 +16,7 @@ ROOT = os.path.dirname(HERE)
 CSRC = os.path.join(HERE, "csrc")
 BUILD = os.path.join(HERE, "_build")
 LIB = os.path.join(HERE, "libexactmap.so")
-SOURCES = ["api.cu", "grid.cu", "tree.cu", "pairs.cu", "integrate.cu", "pseudo.cu", "noalloc.cu",
+SOURCES = ["api.cu", "grid.cu", "tree.cu", "pairs.cu", "integrate.cu", "integrate64.cu", "pseudo.cu", "noalloc.cu",
            "hsolve.cu", "batch.cu", "serve.cu", "inverse.cu", "table.cu", "voronoi.cu", "peaks.cu"]
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 FLAGS = ["-O3", "-lineinfo", "-std=c++17", "-Xcompiler", "-fPIC", "--expt-relaxed-constexpr",

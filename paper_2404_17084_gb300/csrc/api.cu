@@ -174,6 +174,10 @@ int map_init(map_ctx** out, const map_config* cfg) {
     const int r = table_ensure(ctx, nullptr);
     if (r != MAP_OK) { cudaGetLastError(); map_destroy(ctx); return r; }
   }
+  if (ctx->cfg.precision == MAP_FP64) {
+    const int r = fp64_tables(ctx);
+    if (r != MAP_OK) { cudaGetLastError(); map_destroy(ctx); return r; }
+  }
   *out = ctx;
   return MAP_OK;
 }
@@ -211,6 +215,7 @@ void map_destroy(map_ctx* ctx) {
   cudaStreamSynchronize(ctx->cur_stream);
   if (ctx->d_counters) cudaFree(ctx->d_counters);
   if (ctx->d_total) cudaFree(ctx->d_total);
+  if (ctx->d_tables) cudaFree(ctx->d_tables);
   if (ctx->h_stats) cudaFreeHost(ctx->h_stats);
   if (ctx->h_scratch) cudaFreeHost(ctx->h_scratch);
   for (auto& e : ctx->ev) if (e) cudaEventDestroy(e);

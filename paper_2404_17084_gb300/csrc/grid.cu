@@ -56,7 +56,7 @@ __global__ void prep_faces(int64_t nface, const int32_t* __restrict__ fcell, con
   // serves: the radius below is measured from it to the accurate
   // site-relative vertices)
   float mx = 0.f, my = 0.f, mz = 0.f;
-  if (fsph32) {
+  {
     const float sx32 = (float)sx, sy32 = (float)sy, sz32 = (float)sz;
     for (int64_t k = 0; k < L; ++k) {
       const float4 V = v32[fv[b + k]];
@@ -106,9 +106,9 @@ __global__ void prep_faces(int64_t nface, const int32_t* __restrict__ fcell, con
     if (edge64) {
       double rec[9];
       edge_record64(P.x, P.y, P.z, dr, Ax, Ay, Az, Bx, By, Bz, rec);
-      double* E = edge64 + (b + k) * EDGE_STRIDE;
+      double* E = edge64 + (b + k) * EDGE64_STRIDE;
       for (int j = 0; j < 9; ++j) E[j] = rec[j];
-      for (int j = 9; j < EDGE_STRIDE; ++j) E[j] = 0;
+      E[9] = 0.0;
     }
     if (edge32) {
       float rec[12];
@@ -134,17 +134,17 @@ __global__ void prep_faces(int64_t nface, const int32_t* __restrict__ fcell, con
       Ef[0] = make_float4(rec[0], rec[4], rec[1], rec[5]);
       Ef[1] = make_float4(rec[2], rec[6], rec[7], rec[8]);
       Ef[2] = make_float4(rec[3], rec[9], rec[10], rec[11]);
-      if (fsph32) {
-        const float dx = ax32 - mx, dy = ay32 - my, dz = az32 - mz;
-        sr2 = fmaxf(sr2, dx * dx + dy * dy + dz * dz);
-      }
+    }
+    {
+      const float dx = ax32 - mx, dy = ay32 - my, dz = az32 - mz;
+      sr2 = fmaxf(sr2, dx * dx + dy * dy + dz * dz);
     }
     Ax = Bx; Ay = By; Az = Bz;
     ax32 = bx32; ay32 = by32; az32 = bz32;
   }
   // bounding sphere: centre at the vertex mean, radius the largest vertex
   // distance, rounded up (FP32 rounding is far inside the margin)
-  if (fsph32) fsph32[f] = make_float4(mx, my, mz, sqrtf(sr2) * (1.0f + 1e-5f) + 1e-12f);
+  fsph32[f] = make_float4(mx, my, mz, sqrtf(sr2) * (1.0f + 1e-5f) + 1e-12f);
   const double area = 0.5 * acc / n_axis;
   volf[f] = dr * area / 3.0;
   r2f[f] = R2;
@@ -255,15 +255,15 @@ int grid_prepare(map_ctx* ctx, const map_grid* in, PreparedGrid* g, cudaStream_t
   MAP_TRY(ctx_alloc_grid(ctx, g, (void**)&g->face_plane, nf * sizeof(double4_32a)));
   MAP_TRY(ctx_alloc_grid(ctx, g, (void**)&g->face64, nf * sizeof(double4_32a)));
   // FP32 faces for the pair rule's screen; then the records a context's
-  // integral kernel reads: face spheres and FP32 edges for the mixed build
+  // integral kernel reads: face spheres, and FP32 edges for the mixed build
   // (a face whose plane passes within 1e-4 h of a particle takes its side
   // from face64), FP64 edges for the FP64 build
   MAP_TRY(ctx_alloc_grid(ctx, g, (void**)&g->face32, nf * sizeof(float4)));
+  MAP_TRY(ctx_alloc_grid(ctx, g, (void**)&g->fsph32, nf * sizeof(float4)));
   if (ctx->cfg.precision != MAP_FP64) {
-    MAP_TRY(ctx_alloc_grid(ctx, g, (void**)&g->fsph32, nf * sizeof(float4)));
     MAP_TRY(ctx_alloc_grid(ctx, g, (void**)&g->edge32, nl * EDGE_STRIDE * sizeof(float)));
   } else {
-    MAP_TRY(ctx_alloc_grid(ctx, g, (void**)&g->edge64, nl * EDGE_STRIDE * sizeof(double)));
+    MAP_TRY(ctx_alloc_grid(ctx, g, (void**)&g->edge64, nl * EDGE64_STRIDE * sizeof(double)));
   }
   MAP_TRY(ctx_alloc_grid(ctx, g, (void**)&g->site, nc * 3 * sizeof(double)));
   MAP_TRY(ctx_alloc_grid(ctx, g, (void**)&g->vol, nc * sizeof(double)));
@@ -299,12 +299,10 @@ int grid_prepare(map_ctx* ctx, const map_grid* in, PreparedGrid* g, cudaStream_t
   MAP_TRY(ensure_t(ctx, ctx->ws_grid[0], nf, &fcell));
   MAP_TRY(ensure_t(ctx, ctx->ws_grid[1], nf, &volf));
   MAP_TRY(ensure_t(ctx, ctx->ws_grid[2], nf, &r2f));
-  float4* v32 = nullptr;
-  if (g->fsph32) {
-    MAP_TRY(ensure_t(ctx, ctx->ws_grid[3], nv, &v32));
-    vert32<<<nblk(nv, tpb), tpb, 0, s>>>(nv, g->vx, g->vy, g->vz, v32); ++ctx->launches;
-    CUDA_TRY(cudaGetLastError());
-  }
+  float4* v32;
+  MAP_TRY(ensure_t(ctx, ctx->ws_grid[3], nv, &v32));
+  vert32<<<nblk(nv, tpb), tpb, 0, s>>>(nv, g->vx, g->vy, g->vz, v32); ++ctx->launches;
+  CUDA_TRY(cudaGetLastError());
   face_cells<<<(unsigned)blocks, tpb, 0, s>>>(nc, g->cell_face_off, fcell); ++ctx->launches;
   CUDA_TRY(cudaGetLastError());
   prep_faces<<<nblk(nf, tpb), tpb, 0, s>>>(nf, fcell, g->face_vert_off, g->face_vert, g->face_plane, g->vx, g->vy,

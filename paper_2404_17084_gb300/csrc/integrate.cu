@@ -1,37 +1,30 @@
 // Pair integrals and cell sums (Section II-B, Eq. 1-3).
 //
-// Persistent kernel, one warp per cell at a time: a warp pulls a cell from a
-// device work queue and takes the cell's pairs 32 at a time, one pair per
-// lane.  Warps share nothing and never wait for one another.  The cell's
-// site-relative face planes and edge records are read straight from global
-// memory: every lane reads the same record, so each read is one broadcast
-// transaction, served from L1 after the first block of pairs.
+// Persistent kernel, one warp per work item (a cell's pairs, or a slice of
+// them) at a time: a warp pulls an item from a device work queue and takes its
+// pairs 32 at a time, one pair per lane.  Warps share nothing and never wait
+// for one another.
 //
-// For each face (r0 from the plane; the inside flag) and each directed edge
-// of it (R0 and the along-edge coordinates of the vertices), every lane splits
-// its edge integral K'_e into pieces -- at most one inner piece, two middle
-// pieces and two pieces beyond the support -- as (r0, R0, lo, hi), the sign
-// s_f s_e folded into the interval direction.  The pieces beyond the support
+// For each face (r0 from the plane; the inside flag) a lane whose face can
+// reach its support queues the face's edges as (pair, edge) records.  The
+// warp splits 32 records at a time, each edge integral K'_e into pieces -- at
+// most one inner piece, two middle pieces and two pieces beyond the support --
+// as (r0, R0, lo, hi) and the sign s_f s_e.  The pieces beyond the support
 // (-r0 E(r0) dPhi, one atan2 for both) are added by the lane itself.  Inner
 // and middle pieces are pushed onto two per-warp stacks, one per kind;
 // whenever a stack holds 32 pieces the whole warp evaluates them together
 // (every lane the same code), so the costly evaluations run with all lanes
-// busy; the stacks carry over from edge to edge and are flushed after the
-// last face.  Each result is added to its owner lane's compensated (Kahan)
-// accumulator, lanes with the same owner in turn, so the order of additions
-// is fixed and every result is bit-reproducible.
-// (Mixed build: a face whose plane passes within 1e-4 h of the particle has
-// its side and distance taken from the FP64 plane and position; its edges
-// then run through the FP32 pipeline like any other.)
+// busy; the stacks are flushed after the last face.
+// A face whose plane passes within 1e-4 h of the particle has its side and
+// distance taken from the FP64 plane and position; its edges then run through
+// the FP32 pipeline like any other.
 //
 // Per pair: f_ai = [inside] + sum_f sum_e s_f s_e K'_e (see wedge.cuh).
 // M_i = sum_a m_a f_ai is accumulated in FP64 and reduced across the warp;
 // rho_i = M_i / V_i.
 //
-// That is the FP64 build's kernel (pair_integrals).  The mixed build's kernel
-// (pair_integrals_mixed) adds a level of compaction between the face loop and
-// the edges: only a lane whose face can reach its support queues the face's
-// edges, as (pair, edge) records that the warp then splits 32 at a time.
+// This file holds the mixed build's kernel and what every build shares;
+// integrate64.cu holds the FP64 build's, table.cu the table variant's.
 #include <cub/cub.cuh>
 #include <type_traits>
 
@@ -40,10 +33,6 @@
 
 namespace {
 
-template <typename T> struct Vec4;
-template <> struct Vec4<float> { typedef float4 type; };
-template <> struct Vec4<double> { typedef double4_32a type; };
-
 // Mixed build: a face whose plane passes within TAU (in units of h) of the
 // particle has its side and distance decided in FP64: FP32 rounding (~1e-7 h)
 // could otherwise put the particle on the wrong side of the plane; with the
@@ -51,24 +40,10 @@ template <> struct Vec4<double> { typedef double4_32a type; };
 // (they are smooth in r0, and continuous as the particle crosses the plane).
 // A separate FP64 evaluation of such faces was measured: every cell of a
 // 2^18 clumpy snapshot agreed with it and with the FP64 build to the same
-// 3.1e-6, and the FP64 path's registers cost the kernel 15%.  Exact zeros (particle
-// exactly on a plane or edge line) are moved to +EPS on the inner side in the
-// FP64 build: the integral is continuous in the particle position, and
-// treating every exact zero as 'inside' is one consistent displacement of the
-// particle into the cell.
+// 3.1e-6, and the FP64 path's registers cost the kernel 15%.
 constexpr float TAU = 1e-4f;
-constexpr double EPS = 1e-12;
 constexpr unsigned FULL = 0xffffffffu;
 constexpr int LCAP = 96;  // stack depth: < 32 left after a drain + up to 2 pieces per lane
-
-// Exclusive warp prefix sum of v in {0, 1, 2} (two ballots); returns the
-// warp total in *tot.
-__device__ __forceinline__ int warp_excl2(int v, int* tot) {
-  const unsigned lt = (1u << (threadIdx.x & 31)) - 1u;
-  const unsigned b0 = __ballot_sync(FULL, v & 1), b1 = __ballot_sync(FULL, v & 2);
-  *tot = __popc(b0) + 2 * __popc(b1);
-  return __popc(b0 & lt) + 2 * __popc(b1 & lt);
-}
 
 // One edge record (EDGE_STRIDE words, 16-byte aligned) in vector loads:
 // e0..e2 the in-plane edge normal m, e3 its offset delta, e4..e6 the edge
@@ -81,90 +56,47 @@ __device__ __forceinline__ void load_edge(const float* E, float& e0, float& e1, 
   const float4 c = __ldg(reinterpret_cast<const float4*>(E) + 2);
   e0 = a.x; e4 = a.y; e1 = a.z; e5 = a.w; e2 = b.x; e6 = b.y; e7 = b.z; e8 = b.w; e3 = c.x;
 }
-__device__ __forceinline__ void load_edge(const double* E, double& e0, double& e1, double& e2, double& e3,
-                                          double& e4, double& e5, double& e6, double& e7, double& e8) {
-  const double2 a = reinterpret_cast<const double2*>(E)[0], b = reinterpret_cast<const double2*>(E)[1];
-  const double2 c = reinterpret_cast<const double2*>(E)[2], d = reinterpret_cast<const double2*>(E)[3];
-  const double2 f = reinterpret_cast<const double2*>(E)[4];
-  e0 = a.x; e1 = a.y; e2 = b.x; e3 = b.y; e4 = c.x; e5 = c.y; e6 = d.x; e7 = d.y; e8 = f.x;
-}
 
-// Per-warp piece stacks (inner, middle) and the results' accumulators.
-//
-// FP32: col[o][l] sums the pieces of owner lane o that lane l evaluated, so
-// that in a drain every lane adds into its own column (bank l, no conflicts
-// and no ordering between lanes); after the last drain of a block each owner
-// adds up its row (compensated) and clears it.  Every cell sees its own
-// lane's pieces in program order, so the result is bit-reproducible.
-// FP64: one accumulator per owner, lanes with the same owner adding in turn.
-template <typename T>
+// Per-warp piece stacks (inner, middle) and the results' accumulators:
+// col[o][l] sums the pieces of owner lane o that lane l evaluated, so that in
+// a drain every lane adds into its own column (bank l, no conflicts and no
+// ordering between lanes); after the last drain of a block each owner adds up
+// its row (compensated) and clears it.  Every cell sees its own lane's pieces
+// in program order, so the result is bit-reproducible.
 struct WarpStacks {
-  // FP32 adds the pieces beyond the support in the lane itself (one atan2
-  // per edge); FP64, where an atan2 costs far more than the stacking, stacks
-  // them as a third kind
-  static constexpr int NK = sizeof(T) == 4 ? 2 : 3;
-  static constexpr bool COL = sizeof(T) == 4;
-  typename Vec4<T>::type e[NK][LCAP];  // (r0, R0, lo, hi): inner, middle[, beyond]
-  unsigned char own[NK][LCAP];         // owner lane
-  float col[COL ? 32 : 1][32];         // FP32: [owner][evaluating lane]
-  T acc[COL ? 1 : 32];                 // FP64: per-owner sum of its pieces
-  SnapDesc d;                          // the snapshot of the warp's current cell
+  float4 e[2][LCAP];           // (r0, R0, lo, hi): inner, middle
+  unsigned char own[2][LCAP];  // owner lane, the sign s_f s_e in bit 7
+  float col[32][32];           // [owner][evaluating lane]
+  SnapDesc d;                  // the snapshot of the warp's current cell
 };
 
 // Evaluates the queued pieces: every stack holding 32 or more (all that is
 // left when flush), 32 at a time from the top, and adds each result to its
 // owner lane's accumulator.
-template <typename T, bool MIXED>
-__device__ __forceinline__ void drain(WarpStacks<T>& S, int& cnt0, int& cnt1, int& cnt2, bool flush,
-                                   unsigned& t0, unsigned& t1, unsigned& t2) {
+__device__ __forceinline__ void drain(WarpStacks& S, int& cnt0, int& cnt1, bool flush, unsigned& t0, unsigned& t1) {
   const int lane = threadIdx.x & 31;
   for (;;) {
     int K, n;
     if (cnt1 >= 32 || (flush && cnt1 > 0)) { K = 1; n = cnt1 < 32 ? cnt1 : 32; cnt1 -= n; t1 += n; }
     else if (cnt0 >= 32 || (flush && cnt0 > 0)) { K = 0; n = cnt0 < 32 ? cnt0 : 32; cnt0 -= n; t0 += n; }
-    else if (WarpStacks<T>::NK == 3 && (cnt2 >= 32 || (flush && cnt2 > 0))) {
-      K = 2; n = cnt2 < 32 ? cnt2 : 32; cnt2 -= n; t2 += n;
-    } else {
-      break;
-    }
-    const int base = K == 0 ? cnt0 : (K == 1 ? cnt1 : cnt2);
+    else break;
+    const int base = K == 0 ? cnt0 : cnt1;
     const bool on = lane < n;
-    T v = T(0);
-    int o = 32 + lane;  // a key no owner has, for idle lanes
-    if constexpr (WarpStacks<T>::COL) {
-      // every lane evaluates (an idle lane a copy of the first piece) and
-      // adds its value or 0: no divergent region
-      const int idx = base + (on ? lane : 0);
-      const typename Vec4<T>::type P = S.e[K][idx];
-      o = S.own[K][idx];
-      if (K == 1) v = wedge::piece_mid<T, MIXED>(P.x, P.y, P.z, P.w);
-      else v = wedge::piece_inner<T>(P.x, P.y, P.z, P.w);
-      // FP32 pieces are stacked unfolded, their sign s_f s_e in the owner's bit 7
-      v = __int_as_float(__float_as_int(v) ^ ((o & 0x80) << 24));
-      S.col[o & 31][lane] += on ? v : 0.f;  // this lane's column: no other lane touches it
-      __syncwarp();
-    } else {
-      if (on) {
-        const typename Vec4<T>::type P = S.e[K][base + lane];
-        o = S.own[K][base + lane];
-        if (K == 1) v = wedge::piece_mid<T, MIXED>(P.x, P.y, P.z, P.w);
-        else if (K == 0) v = wedge::piece_inner<T>(P.x, P.y, P.z, P.w);
-        else if constexpr (WarpStacks<T>::NK == 3) v = -P.x * wedge::dphi(P.z, P.w, P.y);  // P.x = c0 (the push)
-      }
-      // lanes holding pieces of the same owner add in turn, in lane order
-      const unsigned grp = __match_any_sync(FULL, o);
-      const int rank = __popc(grp & ((1u << lane) - 1u));
-      for (int r = 0;; ++r) {
-        const bool mine = on && rank == r;
-        if (!__any_sync(FULL, mine)) break;
-        if (mine) S.acc[o] += v;  // FP64: plain sums are ample
-        __syncwarp();
-      }
-    }
+    float v = 0.f;
+    // every lane evaluates (an idle lane a copy of the first piece) and
+    // adds its value or 0: no divergent region
+    const int idx = base + (on ? lane : 0);
+    const float4 P = S.e[K][idx];
+    const int o = S.own[K][idx];
+    if (K == 1) v = wedge::piece_mid<float, true>(P.x, P.y, P.z, P.w);
+    else v = wedge::piece_inner<float>(P.x, P.y, P.z, P.w);
+    v = __int_as_float(__float_as_int(v) ^ ((o & 0x80) << 24));
+    S.col[o & 31][lane] += on ? v : 0.f;  // this lane's column: no other lane touches it
+    __syncwarp();
   }
 }
 
-// FP32: this lane's row of the column accumulators, summed with compensation
+// This lane's row of the column accumulators, summed with compensation
 // (Kahan) in a fixed order and cleared for the next block.  Lane o starts at
 // column o, so the 32 lanes read 32 different banks at every step.
 __device__ __forceinline__ float take_row(float (*col)[32], int o, float& comp) {
@@ -196,217 +128,6 @@ __device__ __forceinline__ float face_r0s(const float4& F, float yx, float yy, f
   return __fsub_rn(__fmul_rn(F.w, hinv), __fmaf_rn(F.x, yx, __fmaf_rn(F.y, yy, __fmul_rn(F.z, yz))));
 }
 
-// COUNT: also tally the work (face tests, edge records, pieces) for the
-// operation count; a separate compilation, as the tally holds registers.
-template <typename T, bool MIXED, int NW, int MINB, bool COUNT>
-__global__ void __launch_bounds__(NW * 32, MINB) pair_integrals(BatchArgs B) {
-  typedef typename Vec4<T>::type V4;
-  __shared__ WarpStacks<T> stacks[NW];
-  const int lane = threadIdx.x & 31;
-  WarpStacks<T>& S = stacks[threadIdx.x >> 5];
-  const SnapDesc& A = S.d;
-  wedge::WorkCount wc;
-  unsigned n_in = 0, n_mid = 0;  // stacked pieces evaluated by this warp
-  unsigned n_out = 0;            // this lane's beyond-support intervals (FP32)
-  unsigned n_out_st = 0;         // stacked beyond-support pieces evaluated by this warp (FP64)
-  int n64 = 0;
-  unsigned n_split = 0;  // middle intervals split at the foot (counted once, evaluated as two pieces)
-  int cur = -1;          // snapshot held in S.d
-  if constexpr (WarpStacks<T>::COL) {
-    for (int r = 0; r < 32; ++r) S.col[r][lane] = 0.f;
-    __syncwarp();
-  }
-
-  const int64_t total = queue_total(B);
-  for (;;) {
-    int64_t g = 0;
-    if (lane == 0) g = (int64_t)atomicAdd(&B.counters[3], 1ULL);
-    g = __shfl_sync(FULL, g, 0);
-    if (g >= total) break;
-    // the snapshot owning queue position g: last j with item_base[j] <= g
-    int jl = 0, jh = B.nsnap - 1;
-    while (jl < jh) {
-      const int jm = (jl + jh + 1) >> 1;
-      if (B.item_base[jm] <= g) jl = jm; else jh = jm - 1;
-    }
-    if (jl != cur) {
-      __syncwarp();
-      const unsigned long long* src = reinterpret_cast<const unsigned long long*>(B.snaps + jl);
-      unsigned long long* dst = reinterpret_cast<unsigned long long*>(&S.d);
-      for (int i = lane; i < (int)(sizeof(SnapDesc) / 8); i += 32) dst[i] = src[i];
-      __syncwarp();
-      cur = jl;
-    }
-    const int64_t it = g - B.item_base[jl];
-    const PairItem item = A.items[it];
-    const int64_t c = item.cell;
-    const V4* __restrict__ face = reinterpret_cast<const V4*>(A.face);
-    const T* __restrict__ edge = reinterpret_cast<const T*>(A.edge);
-    const int64_t f0 = A.cfo[c];
-    const int nf = (int)(A.cfo[c + 1] - f0);
-    const int64_t l0 = A.fvo[f0];
-    const T* __restrict__ ecell = edge + l0 * EDGE_STRIDE;
-    const int nedge = (int)(A.fvo[f0 + nf] - l0);
-    double macc = 0.0;
-    const int64_t pb = item.lo, pe = item.lo + item.cnt;
-    for (int64_t p0 = pb; p0 < pe; p0 += 32) {
-      const int64_t p = p0 + lane;
-      const bool active = p < pe;
-      T yx = T(0), yy = T(0), yz = T(0), hinv = T(0);
-      int32_t a = 0;
-      if (active) {
-        a = A.pair_idx[p];
-        const double hh = A.h[a];
-        const double sx = A.site[3 * c], sy = A.site[3 * c + 1], sz = A.site[3 * c + 2];
-        if (MIXED) {
-          const float hi = 1.0f / (float)hh;
-          yx = (float)(A.x[a] - sx) * hi;
-          yy = (float)(A.y[a] - sy) * hi;
-          yz = (float)(A.z[a] - sz) * hi;
-          hinv = hi;
-        } else {
-          const double hi = 1.0 / hh;
-          yx = (A.x[a] - sx) * hi;
-          yy = (A.y[a] - sy) * hi;
-          yz = (A.z[a] - sz) * hi;
-          hinv = hi;
-        }
-      }
-      if constexpr (!WarpStacks<T>::COL) S.acc[lane] = T(0);
-      bool inside = true;
-      double dacc = 0.0;
-      int cnt0 = 0, cnt1 = 0, cnt2 = 0;  // stack heights (warp-uniform)
-      T osum = T(0), ocmp = T(0);  // this lane's beyond-support terms (compensated)
-      int kb = 0;
-      int pk = -1;  // index of the edge record held in n0..n8
-      T n0, n1, n2, n3, n4, n5, n6, n7, n8;
-      for (int fi = 0; fi < nf; ++fi) {
-        const V4 F = face[f0 + fi];
-        const int ke = (int)(A.fvo[f0 + fi + 1] - l0);
-        const T r0s = F.w * hinv - (F.x * yx + F.y * yy + F.z * yz);
-        bool fin = r0s >= T(0);
-        T r0 = fabs(r0s);
-        if (!MIXED) r0 = r0 > T(EPS) ? r0 : T(EPS);
-        bool inrange = active && r0 < T(2);
-        const T c0f = wedge::c0_of(r0);
-        if (COUNT && active) wc.faces++;
-        inside = inside && fin;
-        if (__any_sync(FULL, inrange)) {
-          if (pk != kb) load_edge(ecell + kb * EDGE_STRIDE, n0, n1, n2, n3, n4, n5, n6, n7, n8);
-          for (int k = kb; k < ke; ++k) {
-            const T e0 = n0, e1 = n1, e2 = n2, e3 = n3, e4 = n4, e5 = n5, e6 = n6, e7 = n7, e8 = n8;
-            // the next record (of this face or the next) loads while this one is used
-            pk = k + 1;
-            if (pk < nedge) load_edge(ecell + pk * EDGE_STRIDE, n0, n1, n2, n3, n4, n5, n6, n7, n8);
-            // R0 = m.(p - v_a) (> 0 inside), along-edge vertex positions
-            const T R0s = (e0 * yx + e1 * yy + e2 * yz) - e3 * hinv;
-            const T base = e4 * yx + e5 * yy + e6 * yz;
-            const bool ein = R0s >= T(0);
-            T R0 = fabs(R0s);
-            if (!MIXED) R0 = R0 > T(EPS) ? R0 : T(EPS);
-            const wedge::EdgeSplit<T> P =
-                wedge::split_edge_flat<T>(r0, R0, e7 * hinv - base, e8 * hinv - base, fin == ein, inrange);
-            const int nin = P.v & 1u, nmid = ((P.v >> 1) & 1u) + ((P.v >> 2) & 1u);
-            const int nout = ((P.v >> 3) & 1u) + ((P.v >> 4) & 1u);
-            if (COUNT && inrange) {
-              wc.edges++;
-              if (P.v) wc.terms++;
-              n_split += P.split;
-            }
-            // push this edge's pieces (warp-aggregated)
-            int t0, t1, t2 = 0;
-            const int o0 = cnt0 + warp_excl2(nin, &t0);
-            const int o1 = cnt1 + warp_excl2(nmid, &t1);
-            const unsigned char ln = (unsigned char)lane;
-            T lo, hi;
-            if (P.v & 1u) { P.get(0, lo, hi); S.e[0][o0] = V4{r0, R0, lo, hi}; S.own[0][o0] = ln; }
-            if (P.v & 2u) { P.get(1, lo, hi); S.e[1][o1] = V4{r0, R0, lo, hi}; S.own[1][o1] = ln; }
-            if (P.v & 4u) {
-              const int q = o1 + ((P.v >> 1) & 1u);
-              P.get(2, lo, hi); S.e[1][q] = V4{r0, R0, lo, hi}; S.own[1][q] = ln;
-            }
-            // beyond the support, in this lane: -c0 (dPhi_left + dPhi_right)
-            // as the argument of the product of the two intervals' numbers
-            // (R0^2 + lo hi) + i (hi - lo) R0 -- each angle lies in
-            // (-pi/2, pi/2) and together they span less than pi -- one atan2
-            // per edge, branch-free (an empty interval contributes 1)
-            if constexpr (WarpStacks<T>::NK == 3) {
-              const int o2 = cnt2 + warp_excl2(nout, &t2);
-              if (P.v & 8u) { P.get(3, lo, hi); S.e[2][o2] = V4{c0f, R0, lo, hi}; S.own[2][o2] = ln; }
-              if (P.v & 16u) {
-                const int q = o2 + ((P.v >> 3) & 1u);
-                P.get(4, lo, hi); S.e[2][q] = V4{c0f, R0, lo, hi}; S.own[2][q] = ln;
-              }
-            } else {
-              T l3, h3, l4, h4;
-              P.get(3, l3, h3);
-              P.get(4, l4, h4);
-              const bool v3 = P.v & 8u, v4 = P.v & 16u;
-              const T R02 = R0 * R0;
-              const T ar = v3 ? R02 + l3 * h3 : T(1), ai = v3 ? (h3 - l3) * R0 : T(0);
-              const T br = v4 ? R02 + l4 * h4 : T(1), bi = v4 ? (h4 - l4) * R0 : T(0);
-              const T re = ar * br - ai * bi, im = ar * bi + ai * br;
-              const T y = -c0f * wedge::xatan2(im, re) - ocmp;
-              const T t = osum + y;
-              ocmp = (t - osum) - y;
-              osum = t;
-              if (COUNT) n_out += nout;
-            }
-            cnt0 += t0;
-            cnt1 += t1;
-            cnt2 += t2;
-            __syncwarp();
-            // evaluate full stacks, 32 pieces at a time from the top
-            if (cnt0 >= 32 || cnt1 >= 32 || cnt2 >= 32)
-              drain<T, MIXED>(S, cnt0, cnt1, cnt2, false, n_in, n_mid, n_out_st);
-          }
-        }
-        kb = ke;
-      }
-      // flush what is left (fewer than 32 of each kind)
-      if (cnt0 || cnt1 || cnt2) drain<T, MIXED>(S, cnt0, cnt1, cnt2, true, n_in, n_mid, n_out_st);
-      __syncwarp();
-      double pieces;
-      if constexpr (WarpStacks<T>::COL) {
-        float comp;
-        const float s = take_row(S.col, lane, comp);
-        pieces = (double)s - (double)comp;
-      } else {
-        pieces = (double)S.acc[lane];
-      }
-      if (active) {
-        const double f = (inside ? 1.0 : 0.0) + dacc + pieces + ((double)osum - (double)ocmp);
-        if (A.frac) A.frac[p] = f;
-        macc += A.m[a] * f;
-      }
-      __syncwarp();
-    }
-    for (int o = 16; o > 0; o >>= 1) macc += __shfl_down_sync(FULL, macc, o);
-    if (lane == 0) A.partial[it] = macc;  // summed per cell by cell_sums
-    __syncwarp();
-  }
-  if (!COUNT) return;
-  // work tally: warp sums, one atomic per warp and counter
-  auto wsum = [](unsigned long long v) {
-    for (int o = 16; o > 0; o >>= 1) v += __shfl_down_sync(FULL, v, o);
-    return v;
-  };
-  const unsigned long long terms = wsum((unsigned long long)wc.terms), faces = wsum((unsigned long long)wc.faces);
-  const unsigned long long edges = wsum((unsigned long long)wc.edges), fp64 = wsum((unsigned long long)n64);
-  const unsigned long long split = wsum((unsigned long long)n_split);
-  const unsigned long long outs = wsum((unsigned long long)n_out);
-  if (lane == 0) {
-    atomicAdd(&B.counters[1], terms);
-    atomicAdd(&B.counters[2], fp64);
-    atomicAdd(&B.counters[8], faces);
-    atomicAdd(&B.counters[9], edges);
-    atomicAdd(&B.counters[10], 2ull * n_in);
-    atomicAdd(&B.counters[11], (unsigned long long)n_mid - split);  // a split interval: one interval, two pieces
-    atomicAdd(&B.counters[12], outs + n_out_st);
-    atomicAdd(&B.counters[13], split);
-  }
-}
-
 // ---------------------------------------------------------------- mixed build
 // The mixed build compacts the work twice.  The face loop runs with one pair
 // per lane; a lane whose face is within its support -- plane within 2h and
@@ -429,7 +150,7 @@ struct MixWarp {
   float4 fpl[FSTAGE];    // the item's face planes (site-relative, FP32)
   float4 fsp[FSTAGE];    // their bounding spheres
   int fend[FSTAGE];      // loop end of each face, relative to the cell's first loop entry
-  WarpStacks<float> st;  // piece stacks, column accumulators, snapshot
+  WarpStacks st;  // piece stacks, column accumulators, snapshot
   uint4 cmb[CCAP];       // (r0 bits, c0 bits, edge record offset in floats, fin << 5 | owner)
   float4 py[2][32];      // per pair: (y.x, y.x, y.y, y.y), (y.z, y.z, 1/h, 1/h), y site-relative in units of h
 };
@@ -439,7 +160,7 @@ template <bool COUNT>
 __device__ __forceinline__ void edge_round(MixWarp& M, const float* __restrict__ ecell, int base, int n, int& cnt0,
                                            int& cnt1, unsigned& n_in, unsigned& n_mid, wedge::WorkCount& wc,
                                            unsigned& n_split, unsigned& n_out) {
-  WarpStacks<float>& S = M.st;
+  WarpStacks& S = M.st;
   const int lane = threadIdx.x & 31;
   __syncwarp();
   const bool on = lane < n;
@@ -518,9 +239,7 @@ __device__ __forceinline__ void edge_round(MixWarp& M, const float* __restrict__
   cnt1 += t1;
   __syncwarp();
   if (cnt0 >= 32 || cnt1 >= 32) {
-    int cnt2 = 0;
-    unsigned n_st = 0;
-    drain<float, true>(S, cnt0, cnt1, cnt2, false, n_in, n_mid, n_st);
+    drain(S, cnt0, cnt1, false, n_in, n_mid);
   }
 }
 
@@ -530,7 +249,7 @@ __global__ void __launch_bounds__(NW * 32, MINB) pair_integrals_mixed(BatchArgs 
   const int lane = threadIdx.x & 31;
   const unsigned lt = (1u << lane) - 1u;
   MixWarp& M = mw[threadIdx.x >> 5];
-  WarpStacks<float>& S = M.st;
+  WarpStacks& S = M.st;
   const SnapDesc& A = S.d;
   wedge::WorkCount wc;
   unsigned n_in = 0, n_mid = 0, n_split = 0, n_out = 0;
@@ -561,12 +280,12 @@ __global__ void __launch_bounds__(NW * 32, MINB) pair_integrals_mixed(BatchArgs 
     const int64_t it = g - B.item_base[jl];
     const PairItem item = A.items[it];
     const int64_t c = item.cell;
-    const float4* __restrict__ face = reinterpret_cast<const float4*>(A.face);
+    const float4* __restrict__ face = A.face;
     const float4* __restrict__ fsph = A.fsph;
     const int64_t f0 = A.cfo[c];
     const int nf = (int)(A.cfo[c + 1] - f0);
     const int64_t l0 = A.fvo[f0];
-    const float* __restrict__ ecell = reinterpret_cast<const float*>(A.edge) + l0 * EDGE_STRIDE;
+    const float* __restrict__ ecell = A.edge + l0 * EDGE_STRIDE;
     const double sx = A.site[3 * c], sy = A.site[3 * c + 1], sz = A.site[3 * c + 2];
     const bool staged = nf <= FSTAGE;
     if (staged) {
@@ -647,11 +366,7 @@ __global__ void __launch_bounds__(NW * 32, MINB) pair_integrals_mixed(BatchArgs 
         }
         // what is left: fewer than 32 records, then fewer than 32 pieces of each kind
         if (cntc) edge_round<COUNT>(M, ecell, 0, cntc, cnt0, cnt1, n_in, n_mid, wc, n_split, n_out);
-        if (cnt0 || cnt1) {
-          int cnt2 = 0;
-          unsigned n_st = 0;
-          drain<float, true>(S, cnt0, cnt1, cnt2, true, n_in, n_mid, n_st);
-        }
+        if (cnt0 || cnt1) drain(S, cnt0, cnt1, true, n_in, n_mid);
         __syncwarp();
         float comp;
         const float rs = take_row(S.col, lane, comp);
@@ -710,20 +425,6 @@ int launch_mixed(map_ctx* ctx, const BatchArgs& B, cudaStream_t s) {
   auto kern = pair_integrals_mixed<NW, MINB, COUNT>;
   int per_sm = 0;
   MAP_TRY((mixed_per_sm<NW, MINB, COUNT>(&per_sm, nullptr)));
-  int64_t blocks = (int64_t)per_sm * ctx->sm_count;
-  const int64_t need = (B.total + NW - 1) / NW;
-  if (blocks > need) blocks = need > 0 ? need : 1;
-  kern<<<(unsigned)blocks, NW * 32, 0, s>>>(B); ++ctx->launches;
-  CUDA_TRY(cudaGetLastError());
-  return MAP_OK;
-}
-
-template <typename T, bool MIXED, int NW, int MINB, bool COUNT = false>
-int launch(map_ctx* ctx, const BatchArgs& B, cudaStream_t s) {
-  auto kern = pair_integrals<T, MIXED, NW, MINB, COUNT>;
-  int per_sm = 0;
-  CUDA_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, NW * 32, 0));
-  if (per_sm < 1) per_sm = 1;
   int64_t blocks = (int64_t)per_sm * ctx->sm_count;
   const int64_t need = (B.total + NW - 1) / NW;
   if (blocks > need) blocks = need > 0 ? need : 1;
@@ -822,10 +523,8 @@ int integrals_enqueue(map_ctx* ctx, const BatchArgs& B, int variant, cudaStream_
       case 3: MAP_TRY((launch_mixed<8, 2>(ctx, B, s))); break;
       default: MAP_TRY((launch_mixed<4, 5>(ctx, B, s))); break;
     }
-  } else if (count) {
-    MAP_TRY((launch<double, false, 4, 4, true>(ctx, B, s)));
   } else {
-    MAP_TRY((launch<double, false, 4, 4>(ctx, B, s)));
+    MAP_TRY(launch_fp64(ctx, B, s));
   }
   if (B.total_cells > 0) {
     cell_sums<<<nblk(B.total_cells, 256), 256, 0, s>>>(B.snaps, B.cell_base, B.nsnap, B.total_cells, B.bad);
@@ -866,9 +565,8 @@ SnapDesc make_desc(map_ctx* ctx, const PreparedGrid* g, const map_particles* p, 
   d.frac = frac;
   d.cell_mass = out->cell_mass;
   d.cell_rho = out->cell_rho;
-  const bool mixed = ctx->cfg.precision != MAP_FP64;  // the table variant reads the FP32 records too
-  d.face = mixed ? (const void*)g->face32 : (const void*)g->face64;
-  d.edge = mixed ? (const void*)g->edge32 : (const void*)g->edge64;
+  d.face = g->face32;
+  d.edge = g->edge32;
   d.face64 = g->face64;
   d.edge64 = g->edge64;
   d.fsph = g->fsph32;

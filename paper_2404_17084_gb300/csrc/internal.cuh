@@ -38,7 +38,7 @@ struct PreparedGrid {
   double4_32a* face64 = nullptr;         // site-relative (nx,ny,nz,d - n.s) [nface]
   float4* face32 = nullptr;          // same, FP32
   float4* fsph32 = nullptr;          // per face: bounding-sphere centre (site-relative) and radius, FP32
-  double* edge64 = nullptr;          // EDGE_STRIDE doubles per loop entry (site-relative); FP64 contexts
+  double* edge64 = nullptr;          // EDGE64_STRIDE doubles per loop entry (site-relative); FP64 contexts
   float* edge32 = nullptr;           // EDGE_STRIDE floats per loop entry, interleaved (m.x, t.x, m.y, t.y), (m.z, t.z, a_A, a_B), (delta); mixed contexts
   double* site = nullptr;            // [3*ncell]
   double* vol = nullptr;             // [ncell]
@@ -62,6 +62,8 @@ struct PreparedGrid {
 // m.(p - v_a) = m.(r - s) - delta > 0 when p is on the inner side),
 // unit direction e (3), eps_a = e.(v_a - s), eps_b = e.(v_b - s), pad (3).
 #define EDGE_STRIDE 12
+// FP64 records: 9 doubles and a pad, 16-byte aligned.
+#define EDGE64_STRIDE 10
 
 // The record of the directed edge from vertex A to vertex B (site-relative
 // positions) of a face with unit outward normal (nx, ny, nz), in FP64, into
@@ -223,6 +225,7 @@ struct map_ctx {
   cudaEvent_t wev = nullptr;         // the caller's stream, before the workers start
   // MAP_TABLE: the table of the pyramid integral (n^3 FP32 texels)
   cudaArray_t tab_arr = nullptr;
+  void* d_tables = nullptr;  // MAP_FP64: the integral kernel's function tables
   cudaTextureObject_t tab_tex = 0;
 };
 
@@ -284,10 +287,10 @@ struct SnapDesc {
   const int64_t* item_off;   // [ncell+1]
   double* partial;           // per item
   int64_t nitems;
-  const void* face;    // site-relative planes: float4 (mixed) or double4 (FP64)
-  const void* edge;    // EDGE_STRIDE floats or doubles per loop entry
+  const float4* face;  // site-relative planes, FP32 (mixed, table)
+  const float* edge;   // EDGE_STRIDE floats per loop entry (mixed, table)
   const double4_32a* face64;
-  const double* edge64;
+  const double* edge64;  // EDGE64_STRIDE doubles per loop entry (FP64)
   const float4* fsph;  // per face: bounding sphere (site-relative centre, radius), FP32
   const int32_t* face_vert;          // loop entries -> vertices (the FP64 faces of the mixed build)
   const double *vx, *vy, *vz;
@@ -394,6 +397,10 @@ int integrals_autotune(map_ctx* ctx, const std::function<int(int, BatchArgs&)>& 
 int table_ensure(map_ctx* ctx, cudaStream_t s);
 void table_free(map_ctx* ctx);
 int launch_table(map_ctx* ctx, const BatchArgs& B, cudaStream_t s);
+// FP64 build: its function tables (built by map_init), and its pair-integral
+// kernel
+int fp64_tables(map_ctx* ctx);
+int launch_fp64(map_ctx* ctx, const BatchArgs& B, cudaStream_t s);
 // Runs fn(worker, j) for j = order[0..n) on the context's workers, each on
 // its own stream and host thread, after the work queued on s; s then waits
 // for all of them.  Returns the first error.  Work is handed out in `order`.

@@ -93,12 +93,12 @@ __global__ void __launch_bounds__(NW * 32, MINB) pair_integrals_table(BatchArgs 
     const int64_t it = g - B.item_base[jl];
     const PairItem item = A.items[it];
     const int64_t c = item.cell;
-    const float4* __restrict__ face = reinterpret_cast<const float4*>(A.face);
+    const float4* __restrict__ face = A.face;
     const float4* __restrict__ fsph = A.fsph;
     const int64_t f0 = A.cfo[c];
     const int nf = (int)(A.cfo[c + 1] - f0);
     const int64_t l0 = A.fvo[f0];
-    const float4* __restrict__ ecell = reinterpret_cast<const float4*>(reinterpret_cast<const float*>(A.edge) +
+    const float4* __restrict__ ecell = reinterpret_cast<const float4*>(A.edge +
                                                                        l0 * EDGE_STRIDE);
     const double sx = A.site[3 * c], sy = A.site[3 * c + 1], sz = A.site[3 * c + 2];
     double macc = 0.0;
