@@ -162,3 +162,31 @@ def test_full_size_build_sampled_cells():
     sub.face_plane = g.face_plane.reshape(-1, 4)[faces]
     sub.vx, sub.vy, sub.vz, sub.site = g.vx, g.vy, g.vz, sites[which]
     compare_cells(sub, ref, tol_v=1e-12)
+
+
+
+def _search_sites(kind):
+    rng = np.random.default_rng(17)
+    if kind == "lattice":  # equal distances, cospherical sites: welds, faces of no area
+        return synth.lattice_particles(4).pos()
+    if kind == "shell":  # a cell of many faces
+        u = rng.normal(size=(40, 3))
+        return np.concatenate([[[0.5, 0.5, 0.5]], 0.5 + 0.3 * u / np.linalg.norm(u, axis=1)[:, None], rng.random((109, 3))])
+    if kind == "dense":  # buckets of hundreds beside empty ones, many rings
+        return np.concatenate([0.3 + 0.002 * rng.random((860, 3)), rng.random((40, 3))])
+    return rng.random((int(kind), 3))  # fewer sites than the nearest list holds, and one or two more
+
+
+@pytest.mark.parametrize("kind", ["1", "2", "31", "33", "34", "lattice", "shell", "dense"])
+def test_cells_at_the_edges_of_the_searches(kind):
+    """Volumes of sampled cells against the oracle's to 1e-9 of themselves (a
+    cell's vertices are good to 1e-12 of its size or better), and all of them
+    fill the cube."""
+    sites = _search_sites(kind)
+    g, kept = gpu_build(sites)
+    assert len(kept) == len(sites)
+    vol, _ = oracle.cell_geometry(g)
+    assert abs(vol.sum() - 1.0) < 1e-11
+    which = np.sort(np.random.default_rng(1).choice(len(sites), min(len(sites), 24), replace=False))
+    ref, _ = oracle.cell_geometry(oracle.VoronoiGrid(oracle.voronoi_cells_of(sites, which), sites[which]))
+    assert np.all(np.abs(vol[which] - ref) < 1e-9 * ref)
