@@ -88,12 +88,11 @@ __device__ __forceinline__ void edge_record64(double nx, double ny, double nz, d
   }
 }
 
-// Octree over a particle set (Morton order, level-synchronous build).
+// Octree over a particle set (Morton order).
 struct DevTree {
   int64_t n = 0;          // particles
   int64_t nnodes = 0;
-  int nlevels = 0;
-  std::vector<int64_t> level_begin;  // host: first node of each level (+ end)
+  std::vector<int64_t> level_begin;  // host: first node of each level (+ end); trees built with sizes only
   // particle arrays in Morton order
   uint64_t* keys = nullptr;
   int32_t* idx = nullptr;             // sorted position -> particle index
@@ -118,7 +117,7 @@ struct DevTree {
   unsigned long long* size_bits = nullptr;  // FP64 bits of the node size (max distance to COM)
   unsigned long long* hmax_bits = nullptr;  // FP64 bits of max h in the subtree
   unsigned long long* bbox_bits = nullptr;  // 6 per node: FP64 bits of (minx,miny,minz) and (maxx,maxy,maxz)
-  float* box32 = nullptr;             // 8 per node: FP32 box rounded outward, largest h rounded up, pad
+  float* box32 = nullptr;             // 8 per node: FP32 box rounded outward, largest h rounded up, link
 };
 
 // A work item of the pair-integral kernel: cnt pairs of one cell, starting
