@@ -137,49 +137,72 @@ __global__ void member_write(int64_t nn, const int32_t* __restrict__ flag, const
   members[pos[i]] = (int32_t)i;
 }
 
-__device__ __forceinline__ double w_m4(double q) {
-  if (q < 1.0) return 1.0 - 1.5 * q * q + 0.75 * q * q * q;
-  if (q < 2.0) { double t = 2.0 - q; return 0.25 * t * t * t; }
-  return 0.0;
-}
-__device__ __forceinline__ double dw_m4(double q) {
-  if (q < 1.0) return -3.0 * q + 2.25 * q * q;
-  if (q < 2.0) { double t = 2.0 - q; return -0.75 * t * t; }
-  return 0.0;
+// The members' centres of mass in the order they are scanned, as FP32 hi/lo
+// pairs: x, y, z rounded to FP32 and the node, then what the rounding left.
+__global__ void member_points(int64_t nm, const int32_t* __restrict__ members, const double* __restrict__ com, float4* hi,
+                              float4* lo) {
+  const int64_t j = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+  if (j >= nm) return;
+  const int32_t b = members[j];
+  const double x = com[3 * (int64_t)b], y = com[3 * (int64_t)b + 1], z = com[3 * (int64_t)b + 2];
+  const float hx = (float)x, hy = (float)y, hz = (float)z;
+  hi[j] = make_float4(hx, hy, hz, __int_as_float(b));
+  lo[j] = make_float4((float)(x - (double)hx), (float)(y - (double)hy), (float)(z - (double)hz), 0.f);
 }
 
 struct NodeSet {
-  int64_t nm;                 // members
-  const int32_t* members;     // node ids
-  const double* com;          // node centre of mass (3 per node)
+  int64_t nm;        // members
+  const float4* hi;  // their points (member_points); with use_kmid grouped by their k_mid ancestor
+  const float4* lo;
+  const double* com;  // node centre of mass (3 per node)
   // k_mid candidates (used when use_kmid)
   int use_kmid;
-  int64_t mid_begin, mid_end; // node id range of level k_mid
-  const int64_t* mid_off;     // per mid node: member range in mid_sorted (size nmid+1)
-  const int32_t* mid_sorted;  // members grouped by their k_mid ancestor
+  int64_t mid_begin, mid_end;  // node id range of level k_mid
+  const int64_t* mid_off;      // per mid node: its range of members (size nmid+1)
 };
 
-__device__ __forceinline__ void acc_member(const double* com, int32_t b, double x, double y, double z, double R2,
-                                           double inv_h, double& s, double& ds) {
-  const double dx = com[3 * b] - x, dy = com[3 * b + 1] - y, dz = com[3 * b + 2] - z;
-  const double r2 = dx * dx + dy * dy + dz * dz;
-  if (r2 >= R2) return;
-  const double q = sqrt(r2) * inv_h;
-  const double w = w_m4(q);
-  s += w;
-  ds += 3.0 * w + q * dw_m4(q);
+// What bounds the solve is latency, each sum a chain of gathers over up to
+// 10^4 members or the members of each flagged level-k_mid node: so a warp
+// gathers the candidates within 2.5 h once, as FP32 offsets in shared memory,
+// and iterates on those; FP64 comes in for one last step of third order (as in
+// the full-resolution solve).  Scanning every candidate in FP64 at every
+// Newton step took 2.1 ms for 927 nodes and 17 ms for 16,000; this takes 0.67
+// and 3.6 ms.
+constexpr int PS_CAP = 512;   // candidates held per warp
+constexpr int PS_WARPS = 4;
+struct PseudoWarp {
+  float x[PS_CAP], y[PS_CAP], z[PS_CAP];
+  int32_t node[PS_CAP];
+};
+constexpr unsigned PFULL = 0xffffffffu;
+
+template <typename V>
+__device__ __forceinline__ V lanes_sum(V v) {
+  for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(PFULL, v, o);
+  return v;
 }
 
-// n(h) and dn/dh at (x, y, z) over the candidates, summed by the 32 lanes of
-// a warp (strided over the members or the level-k_mid nodes) and combined by
-// a butterfly reduction, so that every lane holds the same sums.
-__device__ void set_density(const NodeSet& S, int lane, double x, double y, double z, double rcut, double h, double& n,
-                            double& dn) {
-  const double R2 = 4.0 * h * h, inv_h = 1.0 / h, norm = 1.0 / (MAP_PI * h * h * h);
-  double s = 0.0, ds = 0.0;
-  if (!S.use_kmid) {
-    for (int64_t j = lane; j < S.nm; j += 32) acc_member(S.com, S.members[j], x, y, z, R2, inv_h, s, ds);
-  } else {
+struct PseudoSolve {
+  const NodeSet& S;
+  PseudoWarp& W;
+  int lane;
+  double px, py, pz;                // the node's centre of mass
+  float hx, lx, hy, ly, hz, lz;     // its FP32 hi/lo
+  double rcut;
+  float R = -1.f;  // radius the list covers (-1: none)
+  int n = 0;       // its length; -1: it does not fit, every pass scans
+
+  // f(offset x, y, z, node, valid) over the candidates, 32 at a time, every lane calling
+  template <typename F>
+  __device__ __forceinline__ void scan(F f) const {
+    auto range = [&](int64_t a, int64_t b) {
+      for (int64_t j0 = a; j0 < b; j0 += 32) {
+        const int64_t j = j0 + lane < b ? j0 + lane : b - 1;
+        const float4 H = __ldg(S.hi + j), L = __ldg(S.lo + j);
+        f((H.x - hx) + (L.x - lx), (H.y - hy) + (L.y - ly), (H.z - hz) + (L.z - lz), __float_as_int(H.w), j0 + lane < b);
+      }
+    };
+    if (!S.use_kmid) { range(0, S.nm); return; }
     // the lanes test 32 level-k_mid nodes at a time, then share out the
     // members of each flagged one
     const double rc2 = rcut * rcut;
@@ -187,82 +210,175 @@ __device__ void set_density(const NodeSet& S, int lane, double x, double y, doub
       const int64_t m = m0 + lane;
       bool flag = false;
       if (m < S.mid_end) {
-        const double dx = S.com[3 * m] - x, dy = S.com[3 * m + 1] - y, dz = S.com[3 * m + 2] - z;
+        const double dx = S.com[3 * m] - px, dy = S.com[3 * m + 1] - py, dz = S.com[3 * m + 2] - pz;
         flag = dx * dx + dy * dy + dz * dz < rc2;
       }
-      for (unsigned bal = __ballot_sync(0xffffffffu, flag); bal; bal &= bal - 1) {
+      for (unsigned bal = __ballot_sync(PFULL, flag); bal; bal &= bal - 1) {
         const int64_t k = m0 + (__ffs(bal) - 1) - S.mid_begin;
-        for (int64_t j = S.mid_off[k] + lane; j < S.mid_off[k + 1]; j += 32)
-          acc_member(S.com, S.mid_sorted[j], x, y, z, R2, inv_h, s, ds);
+        range(S.mid_off[k], S.mid_off[k + 1]);
       }
     }
   }
-  for (int o = 16; o > 0; o >>= 1) {
-    s += __shfl_xor_sync(0xffffffffu, s, o);
-    ds += __shfl_xor_sync(0xffffffffu, ds, o);
+
+  __device__ __forceinline__ void gather(float r) {
+    const unsigned lt = (1u << lane) - 1u;
+    const float r2 = r * r * 1.00001f;
+    int c = 0;
+    __syncwarp();
+    scan([&](float x, float y, float z, int node, bool on) {
+      const bool in = on && x * x + y * y + z * z < r2;
+      const unsigned m = __ballot_sync(PFULL, in);
+      const int k = c + __popc(m & lt);
+      if (in && k < PS_CAP) { W.x[k] = x; W.y[k] = y; W.z[k] = z; W.node[k] = node; }
+      c += __popc(m);
+    });
+    __syncwarp();
+    R = r;
+    n = c <= PS_CAP ? c : -1;
   }
-  n = s * norm;
-  dn = -ds * norm * inv_h;
-}
+
+  // a list that covers the support 2h and is not far larger than it
+  __device__ __forceinline__ void cover(float h) {
+    if (2.f * h > 0.999f * R || (n < 0 ? R > 2.6f * h : R > 8.f * h)) gather(2.5f * h);
+  }
+
+  // n(h) and dn/dh, FP32
+  __device__ __forceinline__ void density(float h, float& nn, float& dn) {
+    cover(h);
+    const float ih = 1.0f / h;
+    float s = 0.f, d = 0.f;
+    auto add = [&](float x, float y, float z) {
+      const float dx = x * ih, dy = y * ih, dz = z * ih;
+      const float q2 = dx * dx + dy * dy + dz * dz;
+      if (q2 >= 4.f) return;
+      const float q = sqrtf(q2);
+      float w, dwq;
+      if (q < 1.f) { w = 1.f - 1.5f * q2 + 0.75f * q2 * q; dwq = -3.f * q2 + 2.25f * q2 * q; }
+      else { const float t = 2.f - q; w = 0.25f * t * t * t; dwq = -0.75f * t * t * q; }
+      s += w;
+      d += 3.f * w + dwq;
+    };
+    if (n >= 0)
+      for (int j = lane; j < n; j += 32) add(W.x[j], W.y[j], W.z[j]);
+    else
+      scan([&](float x, float y, float z, int, bool on) { if (on) add(x, y, z); });
+    const float norm = ih * ih * ih * (float)(1.0 / MAP_PI);
+    nn = lanes_sum(s) * norm;
+    dn = -lanes_sum(d) * norm * ih;
+  }
+
+  // sums of w(q), q w'(q) and q^2 w''(q) + 2 q w'(q) at h, FP64 behind an FP32 screen
+  __device__ __forceinline__ void sums64(double h, double& s, double& d, double& e) {
+    const float hf = (float)h, r2 = 4.00004f * hf * hf;
+    cover(hf);
+    const double ih = 1.0 / h;
+    s = d = e = 0.0;
+    auto add = [&](int node) {
+      const double* c = S.com + 3 * (int64_t)node;
+      const double ex = (c[0] - px) * ih, ey = (c[1] - py) * ih, ez = (c[2] - pz) * ih;
+      const double q2 = ex * ex + ey * ey + ez * ez, q = sqrt(q2), q3 = q2 * q;
+      if (q < 1.0) {
+        s += 1.0 - 1.5 * q2 + 0.75 * q3;
+        d += 2.25 * q3 - 3.0 * q2;
+        e += 9.0 * (q3 - q2);
+      } else if (q < 2.0) {
+        const double t = 2.0 - q, t2 = t * t;
+        s += 0.25 * t2 * t;
+        d -= 0.75 * t2 * q;
+        e += 1.5 * t * q * (q - t);
+      }
+    };
+    if (n >= 0) {
+      for (int j = lane; j < n; j += 32)
+        if (W.x[j] * W.x[j] + W.y[j] * W.y[j] + W.z[j] * W.z[j] <= r2) add(W.node[j]);
+    } else {
+      scan([&](float x, float y, float z, int node, bool on) { if (on && x * x + y * y + z * z <= r2) add(node); });
+    }
+    s = lanes_sum(s);
+    d = lanes_sum(d);
+    e = lanes_sum(e);
+  }
+};
 
 // One warp per output slot holding an accepted node: Newton-Raphson on
 // h = hfact n(h)^(-1/3) from Eq. (9)'s guess, bisection on [h0/16, 16 h0]
 // when it fails, the guess itself when that has no sign change (Section
-// III-C).  The lanes hold identical sums, so the iteration is warp-uniform.
-__global__ void pseudo_h(int64_t nout, const int32_t* __restrict__ node_of_slot, NodeSet S,
+// III-C); then Halley's step on sum_b w = pi hfact^3 in FP64.  The lanes hold
+// identical sums, so the iteration is warp-uniform.
+__global__ void __launch_bounds__(PS_WARPS * 32) pseudo_h(int64_t nout, const int32_t* __restrict__ node_of_slot, NodeSet S,
                          const unsigned long long* __restrict__ size_bits, const int32_t* __restrict__ parent,
                          const int32_t* __restrict__ level, const int64_t* __restrict__ nb, const double* __restrict__ hs,
                          int kmid, double hfact, double* oh) {
+  __shared__ PseudoWarp sw[PS_WARPS];
   const int lane = threadIdx.x & 31;
   const int64_t j = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
   if (j >= nout) return;
   const int32_t nd = node_of_slot[j];
   if (nd < 0) return;  // extracted particle keeps its h
-  const double x = S.com[3 * nd], y = S.com[3 * nd + 1], z = S.com[3 * nd + 2];
+  const double x = S.com[3 * (int64_t)nd], y = S.com[3 * (int64_t)nd + 1], z = S.com[3 * (int64_t)nd + 2];
+  const float hx = (float)x, hy = (float)y, hz = (float)z;
+  PseudoSolve P{S, sw[threadIdx.x >> 5], lane, x, y, z, hx, (float)(x - (double)hx), hy, (float)(y - (double)hy),
+                hz, (float)(z - (double)hz), 0.0};
   const double s_node = bitsd(size_bits[nd]);
   const double g0 = s_node > 0.0 ? hfact * 2.0 * s_node : hs[nb[nd]];
-  double rcut = 0.0;
   if (S.use_kmid) {
     int32_t a = nd;
     while (level[a] > kmid) a = parent[a];
-    rcut = 1.7320508075688772 * bitsd(size_bits[a]);
+    P.rcut = 1.7320508075688772 * bitsd(size_bits[a]);
     const double r2h = 4.0 * hfact * s_node;
-    if (rcut < r2h) {
+    if (P.rcut < r2h) {
       int32_t up = nd;
       for (int k = 0; k < 2 && parent[up] >= 0; ++k) up = parent[up];
-      rcut = 4.0 * hfact * bitsd(size_bits[up]);
+      P.rcut = 4.0 * hfact * bitsd(size_bits[up]);
     }
   }
+  const float hf_s = (float)hfact, hf_lo = (float)(hfact - (double)hf_s), hf3_s = (float)(hfact / 3.0);
   const double lo = g0 / 16.0, hi = g0 * 16.0;
+  const float lo_s = (float)lo, hi_s = (float)hi;
   double h = g0;
-  bool ok = false;
+  bool ok = false, root = true;
+  float h32 = (float)g0;
   for (int it = 0; it < 30; ++it) {
-    double nn, dn;
-    set_density(S, lane, x, y, z, rcut, h, nn, dn);
-    const double f = h - hfact * pow(nn, -1.0 / 3.0);
-    const double fp = 1.0 + hfact / 3.0 * pow(nn, -4.0 / 3.0) * dn;
-    const double hn = h - f / fp;
-    if (!(hn >= lo && hn <= hi)) break;
-    if (fabs(hn - h) < 1e-10 * hn) { h = hn; ok = true; break; }
-    h = hn;
+    float nn, dn;
+    P.density(h32, nn, dn);
+    const float t = rcbrtf(nn);
+    const float f = (h32 - hf_s * t) - hf_lo * t;
+    const float fp = 1.f + hf3_s * (t * t) * (t * t) * dn;
+    const float d = f / fp, hn = h32 - d;
+    if (!(hn >= lo_s && hn <= hi_s)) break;
+    if (fabsf(hn - h32) < 1e-6f * hn) { h = (double)h32 - (double)d; ok = true; break; }
+    h32 = hn;
   }
   if (!ok) {
-    double nn, dn;
-    set_density(S, lane, x, y, z, rcut, lo, nn, dn);
-    const double flo = lo - hfact * pow(nn, -1.0 / 3.0);
-    set_density(S, lane, x, y, z, rcut, hi, nn, dn);
-    const double fhi = hi - hfact * pow(nn, -1.0 / 3.0);
-    if (!(flo < 0.0 && fhi > 0.0)) {
+    auto g = [&](double v) {
+      float nn, dn;
+      P.density((float)v, nn, dn);
+      return v - hfact * rcbrt((double)nn);
+    };
+    if (!(g(lo) < 0.0 && g(hi) > 0.0)) {
       h = g0;
+      root = false;
     } else {
       double a0 = lo, b0 = hi;
       for (int it = 0; it < 200; ++it) {
         const double mid = 0.5 * (a0 + b0);
-        set_density(S, lane, x, y, z, rcut, mid, nn, dn);
-        if (mid - hfact * pow(nn, -1.0 / 3.0) < 0.0) a0 = mid; else b0 = mid;
+        if (g(mid) < 0.0) a0 = mid; else b0 = mid;
         if (b0 - a0 < 1e-12 * mid) break;
       }
       h = 0.5 * (a0 + b0);
+    }
+  }
+  if (root) {
+    // h <- h (1 + u), S' = -d/h, S'' = e/h^2; again while a step is so large that its cube shows
+    const double target = MAP_PI * hfact * hfact * hfact;
+    for (int it = 0; it < 30; ++it) {
+      double s, d, e;
+      P.sums64(h, s, d, e);
+      const double F = s - target;
+      const double u = 2.0 * F * d / (2.0 * d * d - F * e);
+      if (!(fabs(u) < 1e-2)) break;  // S' is 0 (no neighbour inside): the FP32 root stands
+      h += h * u;
+      if (fabs(u) < 2e-6) break;
     }
   }
   if (lane == 0) oh[j] = h;
@@ -360,8 +476,8 @@ int pseudo_run(map_ctx* ctx, const map_particles* full, const map_walk* walk, ma
   const int64_t nm = ctx->h_scratch[0];
   NodeSet S{};
   S.nm = nm;
-  S.members = members;
   S.com = T.com;
+  const int32_t* scanned = members;
   S.use_kmid = nm > ctx->cfg.ngb_bruteforce_max ? 1 : 0;
   int kmid = 0;
   if (S.use_kmid) {
@@ -392,9 +508,17 @@ int pseudo_run(map_ctx* ctx, const map_particles* full, const map_walk* walk, ma
     mid_ranges<<<nblk(nmid + 1, tpb), tpb, 0, s>>>(nm, nmid, kout, moff); ++ctx->launches;
     CUDA_TRY(cudaGetLastError());
     S.mid_off = moff;
-    S.mid_sorted = vout;
+    scanned = vout;
   }
-  pseudo_h<<<nblk(nout * 32, 128), 128, 0, s>>>(nout, node_of_slot, S, T.size_bits, T.parent, T.level, T.begin, T.hs,
+  float4* points;
+  MAP_TRY(ensure_t(ctx, ctx->ws_pairs[2], 2 * nm, &points));
+  S.hi = points;
+  S.lo = points + nm;
+  if (nm > 0) {
+    member_points<<<nblk(nm, tpb), tpb, 0, s>>>(nm, scanned, T.com, points, points + nm); ++ctx->launches;
+    CUDA_TRY(cudaGetLastError());
+  }
+  pseudo_h<<<nblk(nout * 32, PS_WARPS * 32), PS_WARPS * 32, 0, s>>>(nout, node_of_slot, S, T.size_bits, T.parent, T.level, T.begin, T.hs,
                                            kmid, ctx->cfg.hfact, out->h); ++ctx->launches;
   CUDA_TRY(cudaGetLastError());
   return MAP_OK;
