@@ -48,6 +48,13 @@ __global__ void sum_totals(int n, const double* __restrict__ v, double* out) {
 
 constexpr int BATCH_WORKERS = 8;
 
+// the cells of the largest snapshot
+int64_t largest(const std::vector<SnapDesc>& d) {
+  int64_t n = 0;
+  for (const SnapDesc& s : d) n = std::max(n, s.ncell);
+  return n;
+}
+
 int ensure_workers(map_ctx* ctx) {
   if (!ctx->wev) CUDA_TRY(cudaEventCreateWithFlags(&ctx->wev, cudaEventDisableTiming));
   while ((int)ctx->workers.size() < BATCH_WORKERS) {
@@ -343,7 +350,7 @@ int graph_enqueue(map_ctx* ctx, int nsnap, const map_particles* parts, const int
   gphase(ctx, 2, false, bs, capturing);
   MAP_TRY(integrals_enqueue(ctx, B, ctx->tuned[prec], bs));
   gphase(ctx, 2, true, bs, capturing);
-  MAP_TRY(integrals_sum(ctx, d_desc, nsnap, d_tot, bs));
+  MAP_TRY(integrals_sum(ctx, d_desc, nsnap, largest(qd), d_tot, bs));
   sum_totals<<<1, 32, 0, bs>>>(nsnap, d_tot, ctx->d_total); ++ctx->launches;
   CUDA_TRY(cudaGetLastError());
   return MAP_OK;
@@ -800,7 +807,7 @@ int map_batch(map_ctx* ctx, int nsnap, const map_particles* parts, const int* gr
     int rc = integrals_upload(ctx, qd.data(), ibase.data(), base.data(), nsnap, d_desc, d_ibase, d_cbase,
                               ctx->bstream);
     if (rc == MAP_OK) rc = integrals_enqueue(ctx, B, variant, ctx->bstream);
-    if (rc == MAP_OK) rc = integrals_sum(ctx, d_desc, nsnap, d_tot, ctx->bstream);
+    if (rc == MAP_OK) rc = integrals_sum(ctx, d_desc, nsnap, largest(qd), d_tot, ctx->bstream);
     cudaGraph_t graph = nullptr;
     const cudaError_t ce = cudaStreamEndCapture(ctx->bstream, &graph);
     if (rc != MAP_OK || ce != cudaSuccess) {

@@ -384,7 +384,8 @@ int integrals_enqueue(map_ctx* ctx, const BatchArgs& B, int variant, cudaStream_
 // Launch geometry of shape v of the mixed kernel on the context's device:
 // warps per CTA, CTAs per SM launched, registers per thread.
 int integrals_shape(map_ctx* ctx, int v, int* warps, int* ctas, int* regs);
-int integrals_sum(map_ctx* ctx, const SnapDesc* d_desc, int nsnap, double* totals, cudaStream_t s);
+// (max_cells: the largest snapshot's cells; the snapshots' item partials are overwritten)
+int integrals_sum(map_ctx* ctx, const SnapDesc* d_desc, int nsnap, int64_t max_cells, double* totals, cudaStream_t s);
 // Times every (work-item target, launch shape) pair on the call's inputs and
 // keeps the fastest (ctx->tuned[MAP_MIXED], ctx->item_target).  rebuild(T, B)
 // rebuilds the work items for target T and returns the launch arguments;
