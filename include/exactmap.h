@@ -254,12 +254,13 @@ int map_copy_pairs(map_ctx* ctx, int64_t* pair_off, int32_t* pair_idx, double* p
  * list gets 0.
  *
  * The first call after a mapping builds a particle-major copy of its pair
- * list (cell and f_ai of every pair, 12 bytes per pair, plus 12 bytes per
- * particle), kept by the context until the next mapping call; later calls
- * with other cell values reuse it.  The build's sort workspace (about 20
- * bytes per pair) also stays with the context, for the next mapping's build,
- * until map_destroy.  Asynchronous on stream (ordered after the mapping
- * call like every call of the context).
+ * list (cell and f_ai of every pair, 12 bytes per pair, and padding of at most
+ * 16 pairs per particle, plus 48 bytes per particle and 12 per cell), kept by
+ * the context until the next mapping call; later calls with other cell
+ * values reuse it.  The build's sort workspace (about 12 bytes per pair) also
+ * stays with the context, for the next mapping's build, until map_destroy.
+ * Asynchronous on stream (ordered after the mapping call like every call of
+ * the context).
  * Errors: MAP_EINVAL (NULL pointer; no single mapping call with per-pair
  * integrals in this context: map_batch and the server keep none; n is not
  * that call's particle count; 2^32 or more pairs), MAP_ENOMEM, MAP_ECUDA. */

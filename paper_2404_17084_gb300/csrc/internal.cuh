@@ -152,7 +152,7 @@ struct map_ctx {
   DevBuf ws_grid[4];                   // grid preparation: face -> cell, per-face volume term and radius^2,
                                        // FP32 vertex copies
   DevBuf ws_vor[23];                   // grid construction: buckets, cell slots, CSR arrays
-  DevBuf ws_inv[13];                   // particle-major copy of the pair list (inverse mapping, Eq. 4)
+  DevBuf ws_inv[15];                   // particle-major copy of the pair list (inverse mapping, Eq. 4)
   DevBuf cub_tmp;
   DevTree tree;
   int64_t node_cap0 = 0;  // > 0: octree node arrays start at this capacity (a context whose workspace is fixed)
@@ -169,11 +169,13 @@ struct map_ctx {
   // ascending cell order within a particle), built by the first inverse
   // mapping after the call
   bool inv_ready = false;
-  const int64_t* inv_off = nullptr;   // [last_npart+1]
+  const int64_t* inv_off = nullptr;   // [last_npart+1], by place
   const int32_t* inv_cell = nullptr;  // per entry: the Morton rank of its cell's site
   const double* inv_frac = nullptr;
+  const int64_t* inv_base = nullptr;  // first entry of each work item
   const int32_t* inv_morton = nullptr; // [last_ncell]: cells in Morton order of their sites
-  const int32_t* inv_order = nullptr; // particles by decreasing entry count
+  const int32_t* inv_order = nullptr; // places on the particles' curve in the order of the work
+  const int32_t* inv_pid = nullptr;   // the particle at each place
   const int64_t* inv_nlong = nullptr; // device: particles summed by a whole warp
   struct PairItem* items = nullptr;  // work items of the pair-integral kernel
   int64_t* item_off = nullptr;       // [ncell+1]: items of cell c

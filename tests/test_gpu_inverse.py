@@ -146,6 +146,58 @@ def test_inverse_clumpy_sampled_particles(precision):
         assert abs(got[a] - want) <= TOL[precision][0] * scale, (a, got[a], want)
 
 
+@pytest.mark.parametrize("n,other", [(1, 0), (31, 0), (33, 40), (1025, 0), (2100, 500)])
+def test_inverse_groups_and_windows(n, other):
+    """Particle counts around a group of 32 and a window of 1024, their lists
+    from one cell to every one (more than 256: summed by a whole warp), 300 cells;
+    with `other` the tree is another particle set's by the time of the call.
+    Bit for bit the sequential fused sum, and an infinite value in a cell that
+    lists no particle reaches none (padding entries are not added)."""
+    L = lib()
+    rng = np.random.default_rng(100 + n)
+    sites = rng.random((300, 3))
+    g = synth.voronoi(sites)
+    x = 0.5 + 0.4 * rng.random((n, 3))
+    h = np.full(n, 0.02)
+    h[n // 2] = 0.12
+    p = synth.Particles(*np.ascontiguousarray(x.T), np.full(n, 1.0 / n))
+    for wide in (False, True):
+        if wide:
+            h[0], x[0] = 0.9, 0.5
+            p = synth.Particles(*np.ascontiguousarray(x.T), p.m)
+        ctx = L.map_init(L.map_config_default(precision=1))
+        try:
+            handle = L.map_grid_upload(ctx, L.grid_to_device(g))
+            dx, dy, dz, m, hh = dev_particles(p, h)
+            mass = torch.empty(g.ncell, dtype=torch.float64, device="cuda")
+            L.map_particles_to_cells(ctx, L.make_particles(dx, dy, dz, m, hh), handle, mass)
+            if other:
+                q = synth.uniform_particles(other, 9)
+                qx, qy, qz, qm, qh = dev_particles(q)
+                L.solve_h(ctx, L.make_particles(qx, qy, qz, qm, qh))
+            v = rng.uniform(-1, 1, g.ncell)
+            outs = []
+            for values in (v, None):
+                if values is None:
+                    off, idx, frac = (a.cpu().numpy() for a in L.map_copy_pairs(ctx, g.ncell))
+                    values = np.where(np.diff(off) == 0, np.inf, v)
+                cv = torch.as_tensor(values, dtype=torch.float64, device="cuda")
+                pv = torch.full((n,), -1.0, dtype=torch.float64, device="cuda")
+                L.map_cells_to_particles(ctx, cv, pv)
+                outs.append(pv.cpu().numpy())
+        finally:
+            L.map_destroy(ctx)
+        if wide:
+            assert np.sum(idx == 0) > 256
+        else:
+            assert np.any(np.diff(off) == 0)
+        sample = np.unique(np.concatenate([[0, n // 2, n - 1], rng.choice(n, min(n, 60), replace=False)]))
+        want = fused_sums(off, idx, frac, v, sample)
+        for got in outs:
+            assert np.array_equal(got[sample], want)
+            assert np.all(np.abs(got - oracle.inverse_map(off, idx, frac, v, n)) <= 1e-13)
+
+
 def test_inverse_errors():
     """A wrong particle count, a batch context (no per-pair integrals kept)
     and a context that has not mapped are refused with MAP_EINVAL."""
