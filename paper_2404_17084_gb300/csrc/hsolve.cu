@@ -238,23 +238,23 @@ __device__ __forceinline__ float add_term(float ox, float oy, float oz, float in
 }
 
 // f(position, offset x, y, z, valid) for list[0, cnt): a lane takes positions
-// lane, lane + 32, ... in that order, HS_MLP of them per round with their
+// lane, lane + 32, ... in that order, MLP of them per round with their
 // loads issued together; every lane calls f, for all of a round's positions.
-template <typename F>
+template <int MLP = HS_MLP, typename F>
 __device__ __forceinline__ void for_list(const HsTree& T, const int32_t* list, int cnt, const HsPoint& p, F f) {
   const int lane = threadIdx.x & 31;
-  for (int j0 = 0; j0 < cnt; j0 += 32 * HS_MLP) {
-    int32_t c[HS_MLP];
-    float2 a[HS_MLP], b[HS_MLP], e[HS_MLP];
+  for (int j0 = 0; j0 < cnt; j0 += 32 * MLP) {
+    int32_t c[MLP];
+    float2 a[MLP], b[MLP], e[MLP];
 #pragma unroll
-    for (int u = 0; u < HS_MLP; ++u) {
+    for (int u = 0; u < MLP; ++u) {
       const int j = j0 + 32 * u + lane;
       c[u] = list[j < cnt ? j : cnt - 1];
       const float2* P = reinterpret_cast<const float2*>(T.split + 6 * (int64_t)c[u]);
       a[u] = __ldg(P); b[u] = __ldg(P + 1); e[u] = __ldg(P + 2);
     }
 #pragma unroll
-    for (int u = 0; u < HS_MLP; ++u) {
+    for (int u = 0; u < MLP; ++u) {
       if (j0 + 32 * u >= cnt) break;
       f(c[u], (a[u].x - p.hx) + (a[u].y - p.lx), (b[u].x - p.hy) + (b[u].y - p.ly),
         (e[u].x - p.hz) + (e[u].y - p.lz), j0 + 32 * u + lane < cnt);
@@ -293,12 +293,12 @@ __device__ __forceinline__ void warp_accum_keep(const HsTree& T, const int32_t* 
 // The same over one chunk of a long list; a lane's candidates with q^2 <
 // keep_q2 are appended to its own column keep[32 i + lane], i < HS_PCAP / 32
 // (nl counts past that when they do not fit).
-template <bool NEWTON>
+template <bool NEWTON, int LONG>
 __device__ __forceinline__ void warp_accum_lane(const HsTree& T, const int32_t* list, int cnt, const HsPoint& p,
                                                 float inv_h, float& s, float& d, int32_t* keep, float keep_q2,
                                                 int& nl) {
   const int lane = threadIdx.x & 31;
-  for_list(T, list, cnt, p, [&](int32_t c, float ox, float oy, float oz, bool on) {
+  for_list<LONG>(T, list, cnt, p, [&](int32_t c, float ox, float oy, float oz, bool on) {
     if (!on) return;
     const float q2 = add_term<NEWTON>(ox, oy, oz, inv_h, s, d);
     if (q2 < keep_q2) {
@@ -402,7 +402,7 @@ __device__ __forceinline__ void for_chunks(const HsTree& T, HsWarp& W, HsBuf& B,
 }
 
 // n(h) and dn/dh for the particle at sorted position k (warp-uniform result).
-template <bool NEWTON>
+template <bool NEWTON, int LONG>
 __device__ __forceinline__ void warp_density(const HsTree& T, HsWarp& W, HsBuf& B, HsOwn& O, int64_t k,
                                              const HsPoint& p, float h, float& n, float& dn) {
   const int lane = threadIdx.x & 31;
@@ -455,7 +455,7 @@ __device__ __forceinline__ void warp_density(const HsTree& T, HsWarp& W, HsBuf& 
     const float kq = cR / h;
     int nl = 0;
     for_chunks(T, W, B, [&](const int32_t* list, int c) {
-      warp_accum_lane<NEWTON>(T, list, c, p, inv_h, s, d, room ? W.pcand : nullptr, kq * kq * 1.00001f, nl);
+      warp_accum_lane<NEWTON, LONG>(T, list, c, p, inv_h, s, d, room ? W.pcand : nullptr, kq * kq * 1.00001f, nl);
     });
     __syncwarp();
     B.cR = -1.f;
@@ -539,7 +539,7 @@ __device__ __forceinline__ void density64(const HsTree& T, HsWarp& W, HsBuf& B, 
   e = warp_total(e);
 }
 
-template <bool MIXED>
+template <bool MIXED, int LONG>
 __global__ void __launch_bounds__(HS_WARPS * 32)
     h_solve_leaves(int64_t n, HsTree T, const double* __restrict__ h0s, double hfact, double* hout, int32_t* route) {
   const float hf_s = (float)hfact, hf3_s = (float)(hfact / 3.0), tol_s = 1e-6f;
@@ -594,7 +594,7 @@ __global__ void __launch_bounds__(HS_WARPS * 32)
       bool ok = false;
       for (int it = 0; it < 30; ++it) {
         float nn, dn;
-        warp_density<true>(T, W, B, O, k, p, hs, nn, dn);
+        warp_density<true, LONG>(T, W, B, O, k, p, hs, nn, dn);
         const float t = rcbrtf(nn);
         float f = hs - hf_s * t;
         f -= hf_lo * t;  // hfact as an FP32 pair
@@ -619,7 +619,7 @@ __global__ void __launch_bounds__(HS_WARPS * 32)
         // inside the mixed build's 1e-6 and the FP64 build's last step
         auto g = [&](double hh) {
           float nn, dn;
-          warp_density<false>(T, W, B, O, k, p, (float)hh, nn, dn);
+          warp_density<false, LONG>(T, W, B, O, k, p, (float)hh, nn, dn);
           return hh - hfact * rcbrt((double)nn);
         };
         // Bisection on [lo, hi] needs g(lo) < 0 < g(hi).  g(h)/h is
@@ -717,10 +717,14 @@ int h_solve_run(map_ctx* ctx, const double* x, const double* y, const double* z,
   const HsTree V{T.xs, T.ys, T.zs, T.split, T.begin, T.end, T.first_child, T.nchild, T.owner, T.idx, T.box32};
   const int64_t warps = (n + HS_WIN - 1) / HS_WIN;
   const unsigned blocks = (unsigned)((warps + HS_WARPS - 1) / HS_WARPS);
-  if (ctx->cfg.precision != MAP_FP64)
-    h_solve_leaves<true><<<blocks, HS_WARPS * 32, 0, s>>>(n, V, h0s, ctx->cfg.hfact, h, route);
-  else
-    h_solve_leaves<false><<<blocks, HS_WARPS * 32, 0, s>>>(n, V, h0s, ctx->cfg.hfact, h, route);
+  // Candidates per lane in flight over a list that outgrew its buffer: a small
+  // set lasts as long as the leaf with the longest list (60,013 particles: 2.24
+  // ms with 4, 2.41 with 2; 262,144: 3.83, 4.31), a large one as long as its
+  // warps take together, and the registers of 4 cost it some (2^20: 11.3, 10.5).
+  const bool mixed = ctx->cfg.precision != MAP_FP64;
+  auto kern = n < (int64_t(1) << 19) ? (mixed ? h_solve_leaves<true, 4> : h_solve_leaves<false, 4>)
+                                     : (mixed ? h_solve_leaves<true, 2> : h_solve_leaves<false, 2>);
+  kern<<<blocks, HS_WARPS * 32, 0, s>>>(n, V, h0s, ctx->cfg.hfact, h, route);
   ++ctx->launches;
   CUDA_TRY(cudaGetLastError());
   return MAP_OK;
