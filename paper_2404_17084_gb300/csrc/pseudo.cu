@@ -166,10 +166,11 @@ struct NodeSet {
 // gathers the candidates within 2.5 h once, as FP32 offsets in shared memory,
 // and iterates on those; FP64 comes in for one last step of third order (as in
 // the full-resolution solve).  Scanning every candidate in FP64 at every
-// Newton step took 2.1 ms for 927 nodes and 17 ms for 16,000; this takes 0.67
-// and 3.6 ms.
-constexpr int PS_CAP = 512;   // candidates held per warp
-constexpr int PS_WARPS = 4;
+// Newton step took 2.1 ms for 927 nodes and 17 ms for 16,000; this takes 0.25
+// and 2.6 ms (with lists of 512 and bisection to 1e-12 before the FP64 step:
+// 0.67 and 3.6 ms, the far nodes' bisections scanning at every step).
+constexpr int PS_CAP = 1024;  // candidates held per warp
+constexpr int PS_WARPS = 2;
 struct PseudoWarp {
   float x[PS_CAP], y[PS_CAP], z[PS_CAP];
   int32_t node[PS_CAP];
@@ -363,7 +364,7 @@ __global__ void __launch_bounds__(PS_WARPS * 32) pseudo_h(int64_t nout, const in
       for (int it = 0; it < 200; ++it) {
         const double mid = 0.5 * (a0 + b0);
         if (g(mid) < 0.0) a0 = mid; else b0 = mid;
-        if (b0 - a0 < 1e-12 * mid) break;
+        if (b0 - a0 < 1e-5 * mid) break;  // the FP64 steps below finish
       }
       h = 0.5 * (a0 + b0);
     }
