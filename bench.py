@@ -150,8 +150,17 @@ OPS = {
     "inner_evals": (96, 6),          # one antiderivative: U, Omega, L, P2..P5
     "mid_intervals_mixed": (200, 14),  # 6-node Gauss-Legendre panel + setup + kappa dPhi
     "mid_split_mixed": (200, 14),    # the second piece of an interval split at the foot
-    "mid_intervals_fp64": (240, 14),  # two closed-form evaluations + kappa dPhi
     "outer_intervals": (45, 2),      # -c0 dPhi (both branches of c0 evaluated)
+}
+# The FP64 build's form (FP64-pipe ops: adds, multiplies and FMAs of the
+# formulas as written, the square roots, arctangents and logarithms included;
+# comparisons, clamps and conversions are integer operations there).
+OPS64 = {
+    "face_tests": 4,                 # r0 = d'/h - n.y
+    "edge_records": 17,              # R0, along-edge ends, s2, s1
+    "inner_evals": 45,               # one end of an inner piece (two per piece)
+    "mid_intervals": 85,             # one middle piece: dOmega, dPhi and r0 R0 [P]
+    "outer_intervals": 13,           # -C dPhi
 }
 
 
@@ -191,14 +200,12 @@ def counted_work(L, torch, precision, device, grids, dev, parts):
         L.map_destroy(ctx)
 
 
-def algorithmic_ops(work: dict, terms: int, mixed: bool):
+def algorithmic_ops(work: dict, terms: int):
     f = m = 0
     units = [("face_tests", work["face_tests"]), ("edge_records", work["edge_records"]),
              ("edge_terms", terms), ("inner_evals", work["inner_evals"]),
              ("outer_intervals", work["outer_intervals"]),
-             ("mid_intervals_mixed" if mixed else "mid_intervals_fp64", work["mid_intervals"])]
-    if mixed:
-        units.append(("mid_split_mixed", work["mid_split"]))
+             ("mid_intervals_mixed", work["mid_intervals"]), ("mid_split_mixed", work["mid_split"])]
     for key, cnt in units:
         f += OPS[key][0] * cnt
         m += OPS[key][1] * cnt
@@ -366,18 +373,16 @@ def run_ours(args):
         fp64 = {"value": st64.n_pairs * world / (ms64 * 1e-3), "ms_per_step": ms64, "steps": 1, "warmup": 0,
                 "integrals_ms": integ64, "phases_ms": {k: round(v, 3) for k, v in phases64.items()}}
         # the FP64 kernel against the measured FP64 FMA rate: the op model of
-        # the FP64 form (closed-form middle pieces), every op on the FP64 pipe
-        # (its divides, square roots and arctangents are FP64 sequences; the
-        # model counts each as one MUFU op, so this bound is a lower one)
+        # the FP64 form, every op on the FP64 pipe
         try:
             h64 = torch.from_numpy(h_fp64).to(dev)  # kept alive through the call
-            terms64, work64 = counted_work(L, torch, L.MAP_FP64, local, g, dev, L.make_particles(x, y, z, m, h64))
-            f64_ops, f64_mufu = algorithmic_ops(work64, terms64, False)
+            _, work64 = counted_work(L, torch, L.MAP_FP64, local, g, dev, L.make_particles(x, y, z, m, h64))
+            f64_ops = sum(OPS64[k] * work64[k] for k in OPS64)
             dfma = L.map_device_peaks(local)["dfma"]
-            frac64 = (f64_ops + f64_mufu) / dfma / (integ64 * 1e-3)
-            fp64["roofline"] = {"bound": "fp64", "kernel": "pair_integrals<double>", "achieved": frac64 * dfma / 1e12,
+            frac64 = f64_ops / dfma / (integ64 * 1e-3)
+            fp64["roofline"] = {"bound": "fp64", "kernel": "pair_integrals_fp64", "achieved": frac64 * dfma / 1e12,
                                 "peak": dfma / 1e12, "unit": "Tops/s (FP64 FMA issue)", "frac": frac64,
-                                "ops": int(f64_ops + f64_mufu), "launch_ms": integ64,
+                                "ops": int(f64_ops), "launch_ms": integ64,
                                 "peak_source": "measured: FP64 FMA microbenchmark (map_device_peaks)"}
         except Exception as exc:  # reported, not fatal
             fp64["roofline"] = {"error": str(exc)}
@@ -402,7 +407,7 @@ def run_ours(args):
                  "note": "pyramid integrals interpolated trilinearly (texture unit) in a table of I(r0, R0, phi); "
                          "errors against the FP64 closed form on the same h"}
 
-    f32, mufu = algorithmic_ops(work, terms, True)
+    f32, mufu = algorithmic_ops(work, terms)
     peaks = load_peaks()
     sm_count = torch.cuda.get_device_properties(dev).multi_processor_count
     f_clk = (clocks or {}).get("sm_max_mhz") or peaks.get("sm_max_mhz", 2070.0)
@@ -568,7 +573,7 @@ def run_batch(args):
     del single_mass
     torch.cuda.empty_cache()
     terms, work = counted_work(L, torch, L.MAP_MIXED, local, [g for _, g in snaps], dev, parts)
-    f32, mufu = algorithmic_ops(work, terms, True)
+    f32, mufu = algorithmic_ops(work, terms)
     sm_count = torch.cuda.get_device_properties(dev).multi_processor_count
     f_clk = (clocks or {}).get("sm_max_mhz") or 2070.0
     roof = alu_roofline(L, local, f32, mufu, integ_ms, sm_count, f_clk)
