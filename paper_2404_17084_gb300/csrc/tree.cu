@@ -56,6 +56,47 @@ __global__ void morton_keys(int64_t n, const double* __restrict__ x, const doubl
   idx[i] = (int32_t)i;
 }
 
+// The keys of a small set sorted in one block: a bitonic network over (key,
+// index) in shared memory, P places (a power of two, P >= n), the index as the
+// second key, so that the order is the stable sort's.  Exchanges of up to 32
+// places stay within the warp that owns their 64 places and need no block
+// barrier.  Above 2000 or so the library's radix sort takes 8 passes over the
+// 63 bits, each mostly launch and look-back latency at these sizes: octree of
+// 4096 particles 193 -> 140 us with this; 2000: the same (the library sorts
+// them in one block too); 8192: 206 and 203 us, 16384: 223 and 324 us, so the
+// line lies at 4096.
+constexpr int SORT_THREADS = 1024;
+constexpr int SORT_SMALL = 4096;
+
+__global__ void __launch_bounds__(SORT_THREADS) sort_small(int n, int P, const uint64_t* __restrict__ keys,
+                                                           uint64_t* __restrict__ out, int32_t* __restrict__ idx) {
+  __shared__ uint64_t sk[SORT_SMALL];
+  __shared__ unsigned short si[SORT_SMALL];
+  for (int i = threadIdx.x; i < P; i += SORT_THREADS) {
+    sk[i] = i < n ? keys[i] : ~0ull;  // (padding goes last: a key has 63 bits)
+    si[i] = (unsigned short)i;
+  }
+  __syncthreads();
+  for (int k = 2; k <= P; k <<= 1)
+    for (int j = k >> 1; j > 0; j >>= 1) {
+      for (int t = threadIdx.x; t < P / 2; t += SORT_THREADS) {
+        const int a = 2 * t - (t & (j - 1)), b = a + j;
+        const uint64_t ka = sk[a], kb = sk[b];
+        const unsigned short ia = si[a], ib = si[b];
+        const bool greater = ka > kb || (ka == kb && ia > ib);
+        if (greater == ((a & k) == 0)) {
+          sk[a] = kb; sk[b] = ka;
+          si[a] = ib; si[b] = ia;
+        }
+      }
+      if (j > 32 || (j == 1 && k >= 64)) __syncthreads(); else __syncwarp();
+    }
+  for (int i = threadIdx.x; i < n; i += SORT_THREADS) {
+    out[i] = sk[i];
+    idx[i] = si[i];
+  }
+}
+
 __global__ void gather_sorted(int64_t n, const int32_t* __restrict__ idx, const double* __restrict__ x,
                               const double* __restrict__ y, const double* __restrict__ z,
                               const double* __restrict__ m, const double* __restrict__ h, double* xs, double* ys,
@@ -427,10 +468,17 @@ static int tree_nodes(map_ctx* ctx, const double* x, const double* y, const doub
   if (h) MAP_TRY(ensure_t(ctx, ctx->ws_tree[27], n, &T.hs32));
   morton_keys<<<nblk(n, tpb), tpb, 0, s>>>(n, x, y, z, keys_in, idx_in); ++ctx->launches;
   CUDA_TRY(cudaGetLastError());
-  size_t tmp_bytes = 0;
-  CUDA_TRY(cub::DeviceRadixSort::SortPairs(nullptr, tmp_bytes, keys_in, T.keys, idx_in, T.idx, n, 0, 63, s));
-  MAP_TRY(ctx_ensure(ctx, ctx->cub_tmp, tmp_bytes));
-  CUDA_TRY(cub::DeviceRadixSort::SortPairs(ctx->cub_tmp.p, tmp_bytes, keys_in, T.keys, idx_in, T.idx, n, 0, 63, s));
+  if (n <= SORT_SMALL) {
+    int P = 64;
+    while (P < n) P *= 2;
+    sort_small<<<1, SORT_THREADS, 0, s>>>((int)n, P, keys_in, T.keys, T.idx); ++ctx->launches;
+    CUDA_TRY(cudaGetLastError());
+  } else {
+    size_t tmp_bytes = 0;
+    CUDA_TRY(cub::DeviceRadixSort::SortPairs(nullptr, tmp_bytes, keys_in, T.keys, idx_in, T.idx, n, 0, 63, s));
+    MAP_TRY(ctx_ensure(ctx, ctx->cub_tmp, tmp_bytes));
+    CUDA_TRY(cub::DeviceRadixSort::SortPairs(ctx->cub_tmp.p, tmp_bytes, keys_in, T.keys, idx_in, T.idx, n, 0, 63, s));
+  }
   gather_sorted<<<nblk(n, tpb), tpb, 0, s>>>(n, T.idx, x, y, z, m, h, T.xs, T.ys, T.zs, T.ms, T.hs, T.split,
                                              T.hs32); ++ctx->launches;
   CUDA_TRY(cudaGetLastError());

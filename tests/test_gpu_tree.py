@@ -19,6 +19,34 @@ def _set(kind):
         return np.concatenate([0.5 + 1e-5 * rng.random((300, 3)), rng.random((20, 3))])
     return rng.random((int(kind), 3))
 
+
+def _keys(pos):
+    """Morton keys: 21 bits of each coordinate interleaved, x highest (numpy)."""
+    c = np.minimum(pos * 2.0 ** 21, 2.0 ** 21 - 1).astype(np.uint64)
+    key = np.zeros(len(pos), np.uint64)
+    for b in range(21):
+        for d in range(3):
+            key |= ((c[:, d] >> np.uint64(b)) & np.uint64(1)) << np.uint64(3 * b + 2 - d)
+    return key
+
+
+# the places of the one-block sort (64 to 4096, one exchange per thread up to
+# 2048, two above) and the sizes around its limit
+@pytest.mark.parametrize("n", [1, 2, 63, 64, 65, 1000, 2048, 2049, 4095, 4096, 4097, 5000])
+def test_particles_come_in_stable_morton_order(n):
+    """A source whose r_part covers the cube extracts every particle, listed by
+    Morton position; a quarter of them share their place with another, those in
+    index order."""
+    rng = np.random.default_rng(n)
+    pos = rng.random((n, 3))
+    if n > 3:
+        pos[rng.permutation(n)[: n // 4]] = pos[rng.permutation(n)[: n // 4]]
+    p = synth.Particles(*(np.ascontiguousarray(pos[:, k]) for k in range(3)), np.full(n, 1.0 / n))
+    out = gpu_pseudo(p, np.full(n, 0.1), np.array([0.5, 0.5, 0.5]), r_part=2.0)
+    assert np.all(out["kind"] == 1)
+    assert np.array_equal(out["ident"], np.argsort(_keys(pos), kind="stable"))
+
+
 # words of the maps: 31, 32, 33, 64, 65 positions; a slice of a big node and one
 # particle more; a node of several slices
 @pytest.mark.parametrize("kind", ["1", "16", "17", "31", "32", "33", "64", "65", "4096", "4097", "20000", "coincident",
