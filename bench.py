@@ -170,11 +170,11 @@ OPS64 = {
 # count (the kernel streams the same per-pair data at any size).  It belongs
 # to the kernel as captured: set it to None when the kernel changes.
 INTEGRAL_DRAM_BYTES_PER_PAIR = 49.3
-# DRAM bytes per pair of one inverse-mapping sum (inv_apply, Morton-ordered
-# gather): 449.6 MB read + written for 32,168,427 pairs in ncu on the 2^18
+# DRAM bytes per pair of one inverse-mapping sum (inv_apply, interleaved
+# groups): 417.3 MB read + written for 32,168,427 pairs in ncu on the 2^18
 # clumpy snapshot, scaled by pair count like the figure above; None once the
 # kernel changes.
-INVERSE_DRAM_BYTES_PER_PAIR = 13.97
+INVERSE_DRAM_BYTES_PER_PAIR = 12.97
 
 
 def counted_work(L, torch, precision, device, grids, dev, parts):
