@@ -84,7 +84,11 @@ __global__ void vor_bucket_bounds(int64_t n, int64_t nb, const int32_t* __restri
 }
 
 // the sites' coordinates in bucket order, as FP32 hi/lo pairs: the difference
-// of two of them keeps FP32's relative accuracy
+// of two of them, (hi - hi) + (lo - lo), is good to FP32's relative accuracy and
+// SPLIT_ERR, whichever is larger (lo is rounded at 2^-50, a difference of two
+// lo at 2^-49, on each axis)
+constexpr float SPLIT_ERR = 8e-15f;
+
 __global__ void vor_split(int64_t n, const double* __restrict__ x, const double* __restrict__ y,
                           const double* __restrict__ z, const int32_t* __restrict__ sites, float4* hi, float4* lo) {
   const int64_t k = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
@@ -107,7 +111,8 @@ __device__ __forceinline__ float box_dist2(float px, float py, float pz, int bx0
 }
 
 // merging: drop site i when a site of lower index lies within tol (the buckets
-// that reach within tol of it; FP32 distances decide unless they are close)
+// that reach within tol of it; FP32 distances rule out the sites beyond it by
+// more than their own error, FP64 decides the rest)
 __global__ void vor_merge_flags(int64_t n, const double* __restrict__ x, const double* __restrict__ y,
                                 const double* __restrict__ z, Buckets B, double tol, int64_t* keep) {
   const int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
@@ -118,14 +123,14 @@ __global__ void vor_merge_flags(int64_t n, const double* __restrict__ x, const d
   const int bx = bucket_coord(px, G), by = bucket_coord(py, G), bz = bucket_coord(pz, G);
   const float hx = (float)px, hy = (float)py, hz = (float)pz;
   const float lx = (float)(px - (double)hx), ly = (float)(py - (double)hy), lz = (float)(pz - (double)hz);
-  const float bw = 1.0f / G, t2 = (float)(tol * tol);
+  const float bw = 1.0f / G, reach = ((float)tol + SPLIT_ERR) * 1.00001f, far2 = reach * reach;
   bool k = true;
   for (int dz = -1; dz <= 1 && k; ++dz)
     for (int dy = -1; dy <= 1 && k; ++dy)
       for (int dx = -1; dx <= 1 && k; ++dx) {
         const int cx = bx + dx, cy = by + dy, cz = bz + dz;
         if (cx < 0 || cy < 0 || cz < 0 || cx >= G || cy >= G || cz >= G) continue;
-        if (box_dist2(hx, hy, hz, cx, cx, cy, cz, bw) > t2 * 1.0001f) continue;
+        if (box_dist2(hx, hy, hz, cx, cx, cy, cz, bw) > far2) continue;
         const int64_t b = ((int64_t)cz * G + cy) * G + cx;
         for (int64_t q = B.off[b]; q < B.off[b + 1]; ++q) {
           const float4 H = __ldg(B.hi + q);
@@ -133,7 +138,7 @@ __global__ void vor_merge_flags(int64_t n, const double* __restrict__ x, const d
           if (j >= i) continue;
           const float4 D = __ldg(B.lo + q);
           const float fx = (H.x - hx) + (D.x - lx), fy = (H.y - hy) + (D.y - ly), fz = (H.z - hz) + (D.z - lz);
-          if (fx * fx + fy * fy + fz * fz > t2 * 1.0001f + 1e-37f) continue;
+          if (fx * fx + fy * fy + fz * fz > far2) continue;
           const double ex = x[j] - px, ey = y[j] - py, ez = z[j] - pz;
           if (ex * ex + ey * ey + ez * ez < tol * tol) { k = false; break; }
         }

@@ -190,3 +190,20 @@ def test_cells_at_the_edges_of_the_searches(kind):
     which = np.sort(np.random.default_rng(1).choice(len(sites), min(len(sites), 24), replace=False))
     ref, _ = oracle.cell_geometry(oracle.VoronoiGrid(oracle.voronoi_cells_of(sites, which), sites[which]))
     assert np.all(np.abs(vol[which] - ref) < 1e-9 * ref)
+
+
+@pytest.mark.parametrize("tol", [1e-9, 1e-11, 1e-12, 1e-13])
+def test_merging_decides_every_pair_in_64_bits(tol):
+    """Pairs just inside the tolerance lose one site, pairs just outside it
+    keep both, down to a thousand spacings of the coordinates (tolerance
+    none: the kept sites are the oracle's)."""
+    r = np.random.default_rng(61)
+    n = 2000
+    base = synth.uniform_particles(n, 62).pos() * 0.9 + 0.05
+    u = r.normal(size=(n, 3))
+    far = np.where(np.arange(n) % 2 == 0, r.uniform(0.95, 0.999, n), r.uniform(1.01, 1.2, n))
+    sites = np.concatenate([base, base + (tol * far / np.linalg.norm(u, axis=1))[:, None] * u])
+    ref = oracle.merge_sites(sites, tol)
+    assert 0.4 * n < 2 * n - len(ref) < 0.6 * n
+    _, kept = gpu_build(sites, merge_tol=tol)
+    assert np.array_equal(kept, ref)
