@@ -17,11 +17,12 @@
 //
 // What bounds it is the FP64 pipe (1.8 lanes per clock and SM: an FP64
 // instruction of a warp costs as much as 70 others of its scheduler) and, behind
-// it, the chain of a cell's cuts.  So all that only selects runs in FP32 with a
-// margin that keeps it exact: distances on hi/lo-split coordinates (buckets and
-// sites beyond reach), and each remaining site's plane against all vertices of
-// the current cell, 32 sites at a time, one per lane -- a plane that clears
-// every vertex clears every later, smaller cell too.  About 70 sites come
+// it, the chain of a cell's cuts.  So all that only selects runs in FP32 with
+// margins that keep it exact -- FP32's rounding, and the split's own 8e-15, which
+// counts once sites are closer than 1e-9 or so: distances on hi/lo-split
+// coordinates (buckets and sites beyond reach), and each remaining site's plane
+// against all vertices of the current cell, 32 sites at a time, one per lane -- a
+// plane that clears every vertex clears every later, smaller cell too.  About 70 sites come
 // within reach of a cell and 17 cut it; those 17 take FP64, with lanes over the
 // vertices, the crossing edges and the faces, about 25 FP64 instructions each.
 // One thread per cell with its polyhedra in local memory (3.9 of 32 lanes busy)
@@ -266,15 +267,17 @@ __device__ __forceinline__ void cell_box(CellWarp& W, double sx, double sy, doub
 }
 
 // Whether the plane (n, d) (unit n, FP32) may cut the cell: false only when it
-// clears every vertex by more than FP32's rounding.
-__device__ __forceinline__ bool may_cut(const CellWarp& W, int nv, float nx, float ny, float nz, float d, float rmax) {
+// clears every vertex by more than FP32's rounding and err, what the plane's
+// own error may move it by within rmax of the site.
+__device__ __forceinline__ bool may_cut(const CellWarp& W, int nv, float nx, float ny, float nz, float d, float rmax,
+                                        float err = 0.f) {
   float s = -INFINITY;
 #pragma unroll 4
   for (int i = 0; i < nv; ++i) {
     const float4 v = W.v32[i];
     s = fmaxf(s, fmaf(nx, v.x, fmaf(ny, v.y, nz * v.z)));
   }
-  return s > d - 1e-5f * (rmax + d);
+  return s > d - (1e-5f * (rmax + d) + err);
 }
 
 // Cut the cell by n.x <= d.  Returns 0 when nothing changed, 1 when the cell
@@ -648,12 +651,13 @@ __global__ void __launch_bounds__(VW * 32) vor_cells(int64_t n, const double* __
 
   // The VOR_NEAR nearest sites of the surrounding 27 buckets, one per lane in
   // order of (distance, index).  The site's own bucket comes first and sets a
-  // bound for the others; sites within the bound (FP32, with a margin) gather
-  // in W.key's place 32 at a time and are merged by their FP64 distance.
+  // bound for the others; sites within the bound (FP32, with a margin for its
+  // own error) gather in W.s's place 32 at a time and are merged by their FP64
+  // distance.
   double kd = INFINITY;  // this lane's entry
   int kj = INT32_MAX;
-  double kth = INFINITY;  // the last lane's, and its FP32
-  float kthf = INFINITY;
+  double kth = INFINITY;     // the last lane's
+  float kthf = INFINITY;     // no site within kth has a larger FP32 distance
   int* const queue = reinterpret_cast<int*>(W.s);  // 64 positions
   int nq = 0;
   auto before = [](double da, int ja, double db, int jb) {
@@ -688,7 +692,8 @@ __global__ void __launch_bounds__(VW * 32) vor_cells(int64_t n, const double* __
       if (before(od, oj, kd, kj) == ((lane & h) == 0) && !(oj == kj)) { kd = od; kj = oj; }
     }
     kth = __shfl_sync(VFULL, kd, 31);
-    kthf = (float)kth;
+    const float kr = (sqrtf((float)kth) + SPLIT_ERR) * 1.00001f;
+    kthf = kr * kr;
     const int v = lane + 32 < nq ? queue[lane + 32] : 0;
     __syncwarp();
     if (lane + 32 < nq) queue[lane] = v;
@@ -722,7 +727,7 @@ __global__ void __launch_bounds__(VW * 32) vor_cells(int64_t n, const double* __
         if (f < tot && q != t) {
           const float4 H = __ldg(B.hi + q), D = __ldg(B.lo + q);
           const float fx = (H.x - H0.x) + (D.x - L0.x), fy = (H.y - H0.y) + (D.y - L0.y), fz = (H.z - H0.z) + (D.z - L0.z);
-          in = fx * fx + fy * fy + fz * fz <= kthf * 1.00001f;
+          in = fx * fx + fy * fy + fz * fz <= kthf;
         }
         const unsigned m = __ballot_sync(VFULL, in);
         if (in) queue[nq + __popc(m & ((1u << lane) - 1u))] = (int)q;
@@ -763,6 +768,7 @@ __global__ void __launch_bounds__(VW * 32) vor_cells(int64_t n, const double* __
   // nearest list was full: sites closer than its last entry are done).  A row
   // of buckets along x is one range of sites; lanes find 32 rows' ranges at a
   // time.
+  const float kin = fmaxf(sqrtf((float)kth) * 0.99999f - SPLIT_ERR, 0.f), done2 = kin * kin;  // closer: in the list
   for (int r = kn == VOR_NEAR ? 0 : 2; r <= G && !bad; ++r) {
     // every site outside rings 0..r-1 is at least (r-1) bucket widths away
     const double reach = (r - 1) * bw;
@@ -811,11 +817,13 @@ __global__ void __launch_bounds__(VW * 32) vor_cells(int64_t n, const double* __
           fx = (H.x - H0.x) + (D.x - L0.x); fy = (H.y - H0.y) + (D.y - L0.y); fz = (H.z - H0.z) + (D.z - L0.z);
           d2 = fx * fx + fy * fy + fz * fz;
           j = __float_as_int(H.w);
-          may = d2 < 4.0f * dm::f32(W.rmax2) * 1.00001f && !(r <= 1 && d2 < kthf * 0.99999f);
+          const float far = (2.0f * rmax_of(W.rmax2) + SPLIT_ERR) * 1.00001f;
+          may = d2 < far * far && !(r <= 1 && d2 < done2);
         }
         if (!__any_sync(VFULL, may)) continue;
-        const float il = d2 > 0.f ? rsqrtf(d2) : 0.f;
-        may = may && may_cut(W, W.nv, fx * il, fy * il, fz * il, 0.5f * d2 * il, rmax_of(W.rmax2));
+        // (an offset off by SPLIT_ERR turns the normal by twice that over its length)
+        const float il = d2 > 0.f ? rsqrtf(d2) : 0.f, rmax = rmax_of(W.rmax2);
+        may = may && may_cut(W, W.nv, fx * il, fy * il, fz * il, 0.5f * d2 * il, rmax, SPLIT_ERR * (2.f * rmax * il + 1.f));
         for (unsigned todo = __ballot_sync(VFULL, may); todo; todo &= todo - 1u) {
           const int jk = __shfl_sync(VFULL, j, __ffs(todo) - 1);
           const double ex = x[jk] - sx, ey = y[jk] - sy, ez = z[jk] - sz;

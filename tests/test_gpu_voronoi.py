@@ -207,3 +207,16 @@ def test_merging_decides_every_pair_in_64_bits(tol):
     assert 0.4 * n < 2 * n - len(ref) < 0.6 * n
     _, kept = gpu_build(sites, merge_tol=tol)
     assert np.array_equal(kept, ref)
+
+
+@pytest.mark.parametrize("radius", [1e-3, 1e-9, 2e-10, 1e-10])
+def test_every_site_of_a_shell_is_a_neighbour(radius):
+    """The centre of 40 sites spread evenly over a sphere has 40 faces, at the
+    smallest radii too, where the distances differ by less than FP32 can tell
+    (integers: no tolerance)."""
+    i = np.arange(40) + 0.5
+    z, phi = 1.0 - 2.0 * i / 40, i * np.pi * (3.0 - 5.0 ** 0.5)
+    u = np.stack([np.sqrt(1 - z * z) * np.cos(phi), np.sqrt(1 - z * z) * np.sin(phi), z], 1)
+    c = np.array([0.77, 0.83, 0.71])
+    g, _ = gpu_build(np.concatenate([[c], c + radius * u]))
+    assert g.cell_face_off[1] == 40
