@@ -318,7 +318,10 @@ __global__ void __launch_bounds__(DW * 32, DCTA) pair_integrals_fp64(BatchArgs B
         const double4_32a F = staged ? W.fpl[fi] : A.face64[f0 + fi];
         const float4 Q = staged ? W.fsp[fi] : A.fsph[f0 + fi];
         const int ke = staged ? W.fend[fi] : (int)(A.fvo[f0 + fi + 1] - l0);
-        const double r0s = fma(F.w, hinv, -fma(F.x, yx, fma(F.y, yy, F.z * yz)));
+        // (the product rounded by itself, as y is: a particle on the plane to the
+        // last bit gets 0 and is moved inside with the faces beside it; fused, it
+        // got the rounding of y and a side of its own on each face)
+        const double r0s = __dsub_rn(__dmul_rn(F.w, hinv), fma(F.x, yx, fma(F.y, yy, F.z * yz)));
         const bool fin = !dm::sign(r0s) || r0s == 0.0;
         const double r0 = dm::max2(dm::abs2(r0s), EPS);
         if (COUNT && active) wc.faces++;

@@ -35,3 +35,25 @@ def test_masses_equal_the_oracle(kind, n, h):
     got = gpu_map(g, p, hh, 0)
     assert np.array_equal(got["idx"], ref["idx"])
     assert np.max(np.abs(got["mass"] - ref["mass"])) < 1e-12
+
+
+@pytest.mark.parametrize("h", [0.03, 0.007, 1e-3])
+def test_particles_on_faces_and_edges(h):
+    """A particle on a face of a rectangular cell or on an edge, away from all
+    else, leaves a half or a quarter in each cell around it.  An exact zero is
+    moved inside by 1e-12 h per plane, which moves each fraction by at most
+    2 x 0.7e-12."""
+    product = lambda v: np.stack(np.meshgrid(*[v] * 3, indexing="ij"), -1).reshape(-1, 3)  # noqa: E731
+    g = synth.voronoi(product(np.array([3, 13, 23]) / 32.0))
+    for a in (g.vx, g.vy, g.vz, g.face_plane):  # planes at 8/32 and 18/32, each 5/32 from its sites, to the last bit
+        a[...] = np.round(a * 32) / 32
+    at = product(np.array([3, 8, 13, 18, 23]) / 32.0)
+    on = (at == 0.25) | (at == 0.5625)
+    at = at[on.sum(axis=1) < 3]
+    p = synth.Particles(*(np.ascontiguousarray(at[:, k]) for k in range(3)), np.full(len(at), 1.0 / len(at)))
+    got = gpu_map(g, p, np.full(len(at), h), 0)
+    cell = np.repeat(np.arange(g.ncell), np.diff(got["off"]))
+    r = np.abs(at[got["idx"]] - g.site[cell])
+    want = np.where(np.max(r, axis=1) < 0.16, 0.5 ** np.sum(r > 0.15, axis=1), 0.0)
+    assert np.allclose(np.bincount(got["idx"], want), 1.0)
+    assert np.max(np.abs(got["frac"] - want)) < 1e-11
