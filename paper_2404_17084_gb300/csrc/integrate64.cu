@@ -309,7 +309,9 @@ __global__ void __launch_bounds__(DW * 32, DCTA) pair_integrals_fp64(BatchArgs B
         yz = (__ldg(A.z + a) - sz) * hinv;
       }
       W.py[0][lane] = yx; W.py[1][lane] = yy; W.py[2][lane] = yz; W.py[3][lane] = hinv;
+      // (reach: the support and FP32's error of an offset from y, in units of h)
       const float fx = (float)yx, fy = (float)yy, fz = (float)yz, fh = (float)hinv;
+      const float reach = 2.f + 1e-6f * (fabsf(fx) + fabsf(fy) + fabsf(fz));
       bool inside = true;
       int cr = 0, cm = 0, ci = 0, co = 0;  // stack heights (warp-uniform)
       __syncwarp();
@@ -327,13 +329,14 @@ __global__ void __launch_bounds__(DW * 32, DCTA) pair_integrals_fp64(BatchArgs B
         if (COUNT && active) wc.faces++;
         inside = inside && fin;
         // within the support: the plane, and not the face's bounding sphere
-        // wholly beyond it (an FP32 test: a face that reaches u = 2 - 1e-5 adds
-        // its fifth power, nothing)
+        // wholly beyond it (an FP32 test that keeps every face it is not sure
+        // of: its errors are 3e-7 of |y| and of the sphere's distance in units of
+        // h, of which one is at most the other, 2 and the radius)
         bool near = active && dm::gt(2.0, r0);
         if (near) {
           const float dx = fx - Q.x * fh, dy = fy - Q.y * fh, dz = fz - Q.z * fh;
-          const float rr = 2.f + Q.w * fh;
-          near = dx * dx + dy * dy + dz * dz < rr * rr * 1.00001f;
+          const float rr = reach + Q.w * fh;
+          near = !(dx * dx + dy * dy + dz * dz > rr * rr * 1.00001f);
         }
         const unsigned mn = __ballot_sync(FULL, near);
         if (mn) {

@@ -57,3 +57,27 @@ def test_particles_on_faces_and_edges(h):
     want = np.where(np.max(r, axis=1) < 0.16, 0.5 ** np.sum(r > 0.15, axis=1), 0.0)
     assert np.allclose(np.bincount(got["idx"], want), 1.0)
     assert np.max(np.abs(got["frac"] - want)) < 1e-11
+
+
+def test_small_particles_at_small_faces():
+    """Particles of a 1e-9th of the cells' size just outside the corners of
+    the smallest faces: the distances of such a face are hundreds of h off in
+    FP32.  A particle's fractions add up to 1; each cell places its planes to
+    some 1e-16 / h = 1e-6 h, so to a few 1e-6; 1e-4 leaves a factor of 30."""
+    h = 1e-10
+    g = synth.voronoi(np.random.default_rng(71).random((4000, 3)))
+    v = np.stack([g.vx, g.vy, g.vz], axis=1)
+    at = []
+    for c in range(g.ncell):
+        for f in range(g.cell_face_off[c], g.cell_face_off[c + 1]):
+            w = v[g.face_vert[g.face_vert_off[f]:g.face_vert_off[f + 1]]]
+            mid = w.mean(axis=0)
+            size = np.linalg.norm(w - mid, axis=1)
+            if 1e-7 < size.max() < 0.003 * np.linalg.norm(mid - g.site[c]):
+                at.append(w + 0.7 * h * (w - mid) / size[:, None])
+    at = np.concatenate(at)
+    at = at[np.all((at > 1e-9) & (at < 1.0 - 1e-9), axis=1)]
+    assert len(at) > 200
+    p = synth.Particles(*(np.ascontiguousarray(at[:, k]) for k in range(3)), np.full(len(at), 1.0 / len(at)))
+    got = gpu_map(g, p, np.full(len(at), h), 0)
+    assert np.max(np.abs(np.bincount(got["idx"], got["frac"], len(at)) - 1.0)) < 1e-4
