@@ -37,10 +37,15 @@
 // FP64.  That is the mixed build's h, 5e-8 from the root.  The FP64 build then
 // takes one FP64 step of third order from there: with S(h) = sum_b w(r_ab/h),
 // Eq. (7) is S(h) = pi hfact^3, and Halley's step from the FP64 sums of w,
-// q w' and q^2 w'' + 2 q w' leaves an error of (5e-8)^3.  FP64 sums at every
-// Newton step (4.2 per particle on a pipe at about 1/74 of the FP32 rate, to
-// |dh| < 1e-10 h) took 77 ms at 2^20 clumpy particles; now 22 ms, of which the
-// FP32 solve is 11 ms (mixed: 12.9 ms before; 60,000 particles 5.2 -> 2.0 ms).
+// q w' and q^2 w'' + 2 q w' leaves an error of (5e-8)^3.  FP32 may lead there,
+// not decide: a particle of the FP64 build whose FP32 solve comes near any
+// decision (a bound of the bracket, a sign of g within 1e-4 h, a flat g, values
+// beyond FP32's range) or whose last step does not settle goes on a list that
+// h_solve_exact solves by the same rules with FP64 sums throughout, so that h
+// and its route are FP64's (0.4 ms at 2^20).  FP64 sums at every Newton step
+// (4.2 per particle on a pipe at about 1/74 of the FP32 rate, to |dh| < 1e-10 h)
+// took 77 ms at 2^20 clumpy particles; now 23 ms, of which the FP32 solve is 11
+// ms (mixed: 12.9 ms before; 60,000 particles 5.2 -> 2.0 ms).
 #include "internal.cuh"
 
 namespace {
@@ -471,14 +476,14 @@ __device__ __forceinline__ void warp_density(const HsTree& T, HsWarp& W, HsBuf& 
 
 // FP64 sums of w(q), q w'(q) and q^2 w''(q) + 2 q w'(q) at h over list[0,
 // cnt) around the particle at sorted position k: the candidates an FP32
-// distance screen (1e-5 relative margin) leaves are packed into buf (at least
+// distance screen (1e-5 margin) leaves are packed into buf (at least
 // 64 entries), so that the FP64 terms run with full warps.
 __device__ __forceinline__ void accum64(const HsTree& T, const int32_t* list, int cnt, const HsPoint& p, int64_t k,
                                         double h, int32_t* buf, double& s, double& d, double& e) {
   const int lane = threadIdx.x & 31;
   const unsigned lt = (1u << lane) - 1u;
   const double x = T.xs[k], y = T.ys[k], z = T.zs[k], inv_h = 1.0 / h;
-  const float ih = (float)inv_h;
+  const float ih = (float)inv_h, lim = 2.00001f + 8e-15f * ih, lim2 = lim * lim;  // (8e-15: the split's own error)
   int nb = 0;
   auto drain = [&](int m) {  // the first m (<= 32) of buf
     __syncwarp();
@@ -502,7 +507,7 @@ __device__ __forceinline__ void accum64(const HsTree& T, const int32_t* list, in
   };
   for_list(T, list, cnt, p, [&](int32_t c, float ox, float oy, float oz, bool on) {
     const float dx = ox * ih, dy = oy * ih, dz = oz * ih;
-    const bool in = on && dx * dx + dy * dy + dz * dz <= 4.00004f;
+    const bool in = on && dx * dx + dy * dy + dz * dz <= lim2;
     const unsigned m = __ballot_sync(FULL, in);
     if (in) buf[nb + __popc(m & lt)] = c;
     nb += __popc(m);
@@ -526,7 +531,7 @@ __device__ __forceinline__ void density64(const HsTree& T, HsWarp& W, HsBuf& B, 
   if (B.pk == k && 2.f * hf <= 0.999f * B.pR) {
     accum64(T, W.pcand, B.pn, p, k, h, buf, s, d, e);
   } else {
-    if (2.f * hf > 0.999f * B.R) regather(T, W, B, 2.5f * hf);
+    if (2.f * hf > 0.999f * B.R || B.R > 8.f * hf) regather(T, W, B, 2.5f * hf);
     if (B.expanded) accum64(T, W.cand, (int)B.total, p, k, h, buf, s, d, e);
     else for_chunks(T, W, B, [&](const int32_t* list, int c) {
       // a walk between chunks uses the stack: the packing buffer is local to a chunk
@@ -539,9 +544,59 @@ __device__ __forceinline__ void density64(const HsTree& T, HsWarp& W, HsBuf& B, 
   e = warp_total(e);
 }
 
+// The candidate list of a leaf before anything is gathered.
+__device__ __forceinline__ void list_init(const HsTree& T, int64_t leaf, HsBuf& B) {
+#pragma unroll
+  for (int i = 0; i < 6; ++i) B.q[i] = T.box32[8 * leaf + i];
+  B.R = -1.f;
+  B.nr = 0;
+  B.total = 0;
+  B.rng_done = false;
+  B.expanded = false;
+  B.pk = -1;
+  B.pR = 0.f;
+  B.pn = 0;
+  B.cR = -1.f;
+}
+
+// Bisection's bracket (Eq. 7's g on [lo, hi] = [g0/16, 16 g0]): it needs g(lo) <
+// 0 < g(hi).  g(h)/h is nondecreasing in h (w is nonincreasing in q, so sum_b
+// w(r_ab/h) grows with h), so the sign of g at either end follows from any
+// point between: step from g0 by factors of 2 towards the sign change and
+// bisect the first bracket [a, b] found, evaluating g at lo or hi only when the
+// steps reach them.  False: no sign change.
+template <typename G>
+__device__ __forceinline__ bool bracket_root(double g0, double lo, double hi, G g, double& a, double& b) {
+  a = lo;
+  b = hi;
+  if (g(g0) < 0.0) {
+    a = g0;
+    double y = 2.0 * g0;
+    for (; y < hi; y *= 2.0) {
+      if (g(y) < 0.0) a = y; else { b = y; break; }
+    }
+    return y < hi || g(hi) > 0.0;
+  }
+  b = g0;
+  double y = 0.5 * g0;
+  for (; y > lo; y *= 0.5) {
+    if (g(y) < 0.0) { a = y; break; } else b = y;
+  }
+  return y > lo || g(lo) < 0.0;
+}
+
+// A step of FP32's Newton that FP64's would not take otherwise: the slope is
+// neither flat nor out of range, and the new iterate lies clear of the bounds.
+__device__ __forceinline__ bool clear_step(float fp, float hn, float lo, float hi) {
+  return fabsf(fp) > 0.02f && fabsf(fp) < 50.f &&
+         ((hn > 1.001f * lo && hn < 0.999f * hi) || hn < 0.999f * lo || hn > 1.001f * hi);
+}
+
+// redo, n_redo (FP64 build): the positions left to h_solve_exact.
 template <bool MIXED, int LONG>
 __global__ void __launch_bounds__(HS_WARPS * 32)
-    h_solve_leaves(int64_t n, HsTree T, const double* __restrict__ h0s, double hfact, double* hout, int32_t* route) {
+    h_solve_leaves(int64_t n, HsTree T, const double* __restrict__ h0s, double hfact, double* hout, int32_t* route,
+                   int32_t* redo, unsigned* n_redo) {
   const float hf_s = (float)hfact, hf3_s = (float)(hfact / 3.0), tol_s = 1e-6f;
   const float hf_lo = (float)(hfact - (double)hf_s);
   __shared__ HsWarp sw[HS_WARPS];
@@ -566,17 +621,7 @@ __global__ void __launch_bounds__(HS_WARPS * 32)
     for (int64_t k = a0 + lane; k < a1; k += 32) gmax = fmax(gmax, h0s[k]);
     for (int o = 16; o > 0; o >>= 1) gmax = fmax(gmax, __shfl_xor_sync(FULL, gmax, o));
     HsBuf B;
-#pragma unroll
-    for (int i = 0; i < 6; ++i) B.q[i] = T.box32[8 * (int64_t)L + i];
-    B.R = -1.f;
-    B.nr = 0;
-    B.total = 0;
-    B.rng_done = false;
-    B.expanded = false;
-    B.pk = -1;
-    B.pR = 0.f;
-    B.pn = 0;
-    B.cR = -1.f;
+    list_init(T, L, B);
     HsOwn O;
     O.n = 0;
     const float R0 = 2.5f * (float)gmax;
@@ -592,6 +637,7 @@ __global__ void __launch_bounds__(HS_WARPS * 32)
       const float lo_s = hs / 16.f, hi_s = hs * 16.f;
       double h = 0.0;
       bool ok = false;
+      bool sure = true;  // (FP64 build) FP32 has decided as FP64 would
       for (int it = 0; it < 30; ++it) {
         float nn, dn;
         warp_density<true, LONG>(T, W, B, O, k, p, hs, nn, dn);
@@ -601,6 +647,10 @@ __global__ void __launch_bounds__(HS_WARPS * 32)
         const float fp = 1.f + hf3_s * (t * t) * (t * t) * dn;
         const float d = f / fp;
         const float hn = hs - d;
+        if (!MIXED) {
+          sure = it < 24 && clear_step(fp, hn, lo_s, hi_s);
+          if (!sure) break;
+        }
         if (!(hn >= lo_s && hn <= hi_s)) break;
         if ((hn > hs ? hn - hs : hs - hn) < tol_s * hn) {
           // the converged step is applied in FP64 (the result keeps FP64's
@@ -612,22 +662,19 @@ __global__ void __launch_bounds__(HS_WARPS * 32)
         hs = hn;
       }
       int r = 0;
-      if (!ok) {
-        const double g0 = h0s[k];
-        const double lo = g0 / 16.0, hi = g0 * 16.0;
+      if (!ok && sure) {
+        const double g0 = h0s[k], lo = g0 / 16.0, hi = g0 * 16.0;
         // bisection on the FP32 sums too: the root moves by ~1e-7 relative,
         // inside the mixed build's 1e-6 and the FP64 build's last step
         auto g = [&](double hh) {
           float nn, dn;
           warp_density<false, LONG>(T, W, B, O, k, p, (float)hh, nn, dn);
-          return hh - hfact * rcbrt((double)nn);
+          const double v = hh - hfact * rcbrt((double)nn);
+          if (!MIXED) sure = sure && fabs(v) > 1e-4 * hh && nn < 1e37f;
+          return v;
         };
-        // Bisection on [lo, hi] needs g(lo) < 0 < g(hi).  g(h)/h is
-        // nondecreasing in h (w is nonincreasing in q, so sum_b w(r_ab/h)
-        // grows with h), so the sign of g at either end follows from any
-        // point between: step from h0 by factors of 2 towards the sign change
-        // and bisect the first bracket found, evaluating g at lo or hi only
-        // when the steps reach them.
+        // (bracket_root written out: as a function it cost the mixed build 4% at
+        // 2^20, 12.8 -> 13.3 ms, with g inlined once more)
         double a = lo, b = hi;
         bool bracket = true;
         if (g(g0) < 0.0) {
@@ -648,29 +695,37 @@ __global__ void __launch_bounds__(HS_WARPS * 32)
         if (!bracket) {
           h = g0;
           r = 2;
-        } else {
+        } else if (sure) {
           for (int it = 0; it < 200; ++it) {
             const double mid = 0.5 * (a + b);
             if (g(mid) < 0.0) a = mid; else b = mid;
-            if (b - a < 1e-12 * mid) break;
+            if (!MIXED && !sure) { a = b = mid; break; }  // at the root, as far as FP32 can tell
+            if (b - a < (MIXED ? 1e-12 : 1e-4) * mid) break;
           }
           h = 0.5 * (a + b);
           r = 1;
+          sure = true;
         }
       }
-      if (!MIXED && r != 2) {
+      if (!MIXED && r != 2 && sure) {
         // Halley's step on S(h) - pi hfact^3 (S' = -d/h, S'' = e/h^2), again
-        // while a step is so large that its cube shows
+        // while a step is so large that its cube shows; one that is large or no
+        // number (S' is 0) leaves the particle to h_solve_exact
         const double target = MAP_PI * hfact * hfact * hfact;
+        sure = false;
         for (int it = 0; it < 30; ++it) {
           double s, d, e;
           density64(T, W, B, k, p, h, s, d, e);
           const double F = s - target;
           const double u = 2.0 * F * d / (2.0 * d * d - F * e);  // -dh / h times -1: h <- h (1 + u)
-          if (!(fabs(u) < 1e-2)) break;  // S' is 0 (no neighbour inside): the FP32 root stands
+          if (!(fabs(u) < 1e-2)) break;
           h += h * u;
-          if (fabs(u) < 2e-6) break;
+          if (fabs(u) < 2e-6) { sure = h > h0s[k] / 16.0 && h < h0s[k] * 16.0; break; }
         }
+      }
+      if (!MIXED && !sure) {
+        if (lane == 0) redo[atomicAdd(n_redo, 1u)] = (int32_t)k;
+        continue;
       }
       if (lane == 0) {
         const int32_t a = T.idx[k];
@@ -681,19 +736,88 @@ __global__ void __launch_bounds__(HS_WARPS * 32)
   }
 }
 
-// Initial guess: hfact * side(leaf cube) / count^(1/3), per sorted position.
+// The listed particles of the FP64 build, one per warp, with FP64 sums
+// throughout: Newton to |dh| < 1e-10 h, bisection to 1e-12, the estimate.  At
+// 2^20 clumpy particles it takes 0.43 of the solve's 25.0 ms.
+__global__ void __launch_bounds__(HS_WARPS * 32)
+    h_solve_exact(HsTree T, const double* __restrict__ h0s, double hfact, const int32_t* __restrict__ redo,
+                  const unsigned* __restrict__ n_redo, double* hout, int32_t* route) {
+  __shared__ HsWarp sw[HS_WARPS];
+  HsWarp& W = sw[threadIdx.x >> 5];
+  const int lane = threadIdx.x & 31;
+  const int64_t count = *n_redo, step = (int64_t)gridDim.x * HS_WARPS;
+  for (int64_t i = blockIdx.x * (int64_t)HS_WARPS + (threadIdx.x >> 5); i < count; i += step) {
+    const int64_t k = redo[i];
+    HsBuf B;
+    list_init(T, T.owner[k], B);
+    const HsPoint p = point_of(T, k);
+    auto density = [&](double h, double& nn, double& dn) {
+      double s, d, e;
+      density64(T, W, B, k, p, h, s, d, e);
+      const double ih = 1.0 / h, norm = ih * ih * ih * (1.0 / MAP_PI);
+      nn = s * norm;
+      dn = -(3.0 * s + d) * norm * ih;
+    };
+    const double g0 = h0s[k], lo = g0 / 16.0, hi = g0 * 16.0;
+    double h = g0;
+    bool ok = false;
+    for (int it = 0; it < 30; ++it) {
+      double nn, dn;
+      density(h, nn, dn);
+      const double t = rcbrt(nn), t2 = t * t;
+      const double hn = h - (h - hfact * t) / (1.0 + hfact / 3.0 * t2 * t2 * dn);
+      if (!(hn >= lo && hn <= hi)) break;
+      ok = fabs(hn - h) < 1e-10 * hn;
+      h = hn;
+      if (ok) break;
+    }
+    int r = 0;
+    if (!ok) {
+      auto g = [&](double v) {
+        double nn, dn;
+        density(v, nn, dn);
+        return v - hfact * rcbrt(nn);
+      };
+      double a, b;
+      if (!bracket_root(g0, lo, hi, g, a, b)) {
+        h = g0;
+        r = 2;
+      } else {
+        for (int it = 0; it < 200; ++it) {
+          const double mid = 0.5 * (a + b);
+          if (g(mid) < 0.0) a = mid; else b = mid;
+          if (b - a < 1e-12 * mid) break;
+        }
+        h = 0.5 * (a + b);
+        r = 1;
+      }
+    }
+    if (lane == 0) {
+      const int32_t a = T.idx[k];
+      hout[a] = h;
+      if (route) route[a] = r;
+    }
+    __syncwarp();
+  }
+}
+
+// Initial guess: hfact * side(leaf cube) / count^(1/3), per sorted position
+// (and *n_redo = 0).
 __global__ void h_guess_leaf(int64_t n, const int32_t* __restrict__ owner, const int32_t* __restrict__ lev,
                              const int64_t* __restrict__ nb, const int64_t* __restrict__ ne, double hfact,
-                             double* h0s) {
+                             double* h0s, unsigned* n_redo) {
   int64_t k = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+  if (k == 0) *n_redo = 0u;
   if (k >= n) return;
   int32_t leaf = owner[k];
   double side = ldexp(1.0, -lev[leaf]);
   h0s[k] = hfact * side / cbrt((double)(ne[leaf] - nb[leaf]));
 }
 
-__global__ void gather_h0(int64_t n, const int32_t* __restrict__ idx, const double* __restrict__ h0, double* h0s) {
+__global__ void gather_h0(int64_t n, const int32_t* __restrict__ idx, const double* __restrict__ h0, double* h0s,
+                          unsigned* n_redo) {
   int64_t k = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+  if (k == 0) *n_redo = 0u;
   if (k >= n) return;
   h0s[k] = h0[idx[k]];
 }
@@ -707,11 +831,15 @@ int h_solve_run(map_ctx* ctx, const double* x, const double* y, const double* z,
   DevTree& T = ctx->tree;
   double* h0s;
   MAP_TRY(ensure_t(ctx, ctx->ws_tree[22], n, &h0s));
+  // the FP64 build's list of particles for h_solve_exact and its length, in the
+  // buffers of the unsorted indices and keys, which are done with
+  int32_t* redo = reinterpret_cast<int32_t*>(ctx->ws_tree[1].p);
+  unsigned* n_redo = reinterpret_cast<unsigned*>(ctx->ws_tree[0].p);
   const int tpb = 128;
   if (h0_override)
-    gather_h0<<<nblk(n, tpb), tpb, 0, s>>>(n, T.idx, h0_override, h0s);
+    gather_h0<<<nblk(n, tpb), tpb, 0, s>>>(n, T.idx, h0_override, h0s, n_redo);
   else
-    h_guess_leaf<<<nblk(n, tpb), tpb, 0, s>>>(n, T.owner, T.level, T.begin, T.end, ctx->cfg.hfact, h0s);
+    h_guess_leaf<<<nblk(n, tpb), tpb, 0, s>>>(n, T.owner, T.level, T.begin, T.end, ctx->cfg.hfact, h0s, n_redo);
   ++ctx->launches;
   CUDA_TRY(cudaGetLastError());
   const HsTree V{T.xs, T.ys, T.zs, T.split, T.begin, T.end, T.first_child, T.nchild, T.owner, T.idx, T.box32};
@@ -724,8 +852,14 @@ int h_solve_run(map_ctx* ctx, const double* x, const double* y, const double* z,
   const bool mixed = ctx->cfg.precision != MAP_FP64;
   auto kern = n < (int64_t(1) << 19) ? (mixed ? h_solve_leaves<true, 4> : h_solve_leaves<false, 4>)
                                      : (mixed ? h_solve_leaves<true, 2> : h_solve_leaves<false, 2>);
-  kern<<<blocks, HS_WARPS * 32, 0, s>>>(n, V, h0s, ctx->cfg.hfact, h, route);
+  kern<<<blocks, HS_WARPS * 32, 0, s>>>(n, V, h0s, ctx->cfg.hfact, h, route, redo, n_redo);
   ++ctx->launches;
   CUDA_TRY(cudaGetLastError());
+  if (!mixed) {
+    const unsigned most = (unsigned)ctx->sm_count * 16;
+    h_solve_exact<<<blocks < most ? blocks : most, HS_WARPS * 32, 0, s>>>(V, h0s, ctx->cfg.hfact, redo, n_redo, h, route);
+    ++ctx->launches;
+    CUDA_TRY(cudaGetLastError());
+  }
   return MAP_OK;
 }

@@ -6,7 +6,7 @@ import torch
 
 import oracle
 import synth
-from gpu_helpers import lib
+from gpu_helpers import dev_particles, lib, oracle_h
 
 pytestmark = pytest.mark.gpu
 
@@ -51,3 +51,31 @@ def test_h_and_route_equal_the_oracle(name, precision, tol):
     ref, want = oracle.solve_h(p.x, p.y, p.z, oracle.particle_h_guess(oracle.Tree(p.x, p.y, p.z, p.m)))
     assert np.array_equal(route, want)
     assert np.max(np.abs(h / ref - 1.0)) < tol
+
+
+@pytest.mark.parametrize("kind", ["line", "plane", "pairs"])
+def test_fp64_routes_are_the_oracles(kind):
+    """Sets on which Newton ends near the bracket's bounds or on flat stretches:
+    the FP64 build takes the oracle's route for every particle, and both stop
+    within 1e-10 of the root (2e-10 apart at most)."""
+    L = lib()
+    ctx = L.map_init(L.map_config_default(precision=L.MAP_FP64))
+    try:
+        for seed in range(6):
+            r = np.random.default_rng(80 + seed)
+            u = r.random((3, 4000))
+            if kind == "pairs":
+                u[:, :2000] = np.clip(u[:, 2000:] + 1e-5 * r.normal(size=(3, 2000)), 0.0, 1.0)
+            elif kind == "line":
+                u[1:] = 0.5
+            else:
+                u[2] = 0.25
+            p = synth.Particles(*u, np.full(4000, 1.0 / 4000))
+            x, y, z, m, h = dev_particles(p)
+            route = torch.empty(p.n, dtype=torch.int32, device="cuda")
+            L.solve_h(ctx, L.make_particles(x, y, z, m, h), route)
+            want, want_route = oracle_h(p)
+            assert np.array_equal(route.cpu().numpy(), want_route)
+            assert np.max(np.abs(h.cpu().numpy() / want - 1.0)) < 2e-10
+    finally:
+        L.map_destroy(ctx)
