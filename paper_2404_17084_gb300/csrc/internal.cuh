@@ -88,6 +88,15 @@ __device__ __forceinline__ void edge_record64(double nx, double ny, double nz, d
   }
 }
 
+// Whether FP64 takes a step of FP32's Newton (from h, of slope gp) as FP32 does:
+// within the bracket (lo, hi) or out of it by more than the step may be off.
+// FP32's sums leave 3e-7 in g / h and 2e-6 in the slope.
+__device__ __forceinline__ bool clear_step(float h, float step, float gp, float lo, float hi) {
+  const float hn = h - step, e = (1e-6f * h + 8e-6f * fabsf(step)) / fabsf(gp);
+  if (!(fabsf(gp) < 50.f)) return false;
+  return (hn > 1.001f * lo + e && hn < 0.999f * hi - e && e < 0.01f * hn) || hn < 0.999f * lo - e || hn > 1.001f * hi + e;
+}
+
 // Octree over a particle set (Morton order).
 struct DevTree {
   int64_t n = 0;          // particles

@@ -165,7 +165,14 @@ struct NodeSet {
 // 10^4 members or the members of each flagged level-k_mid node: so a warp
 // gathers the candidates within 2.5 h once, as FP32 offsets in shared memory,
 // and iterates on those; FP64 comes in for one last step of third order (as in
-// the full-resolution solve).  Scanning every candidate in FP64 at every
+// the full-resolution solve).  FP32 leads there and decides only what is clear
+// in FP32: a node that comes near a bound of the bracket, a sign of g within
+// 1e-4 h, a flat g, or neighbours at a distance that the hi/lo split does not
+// resolve (h < 1e-8), or whose last step does not settle, is solved with FP64
+// sums throughout.  A node's size may be 1e-17 (one particle's rounded centre of
+// mass), where n(h) leaves FP32's range: there only a node by itself is clear,
+// and its g is known.
+// Scanning every candidate in FP64 at every
 // Newton step took 2.1 ms for 927 nodes and 17 ms for 16,000; this takes 0.25
 // and 2.6 ms (with lists of 512 and bisection to 1e-12 before the FP64 step:
 // 0.67 and 3.6 ms, the far nodes' bisections scanning at every step).
@@ -176,6 +183,8 @@ struct PseudoWarp {
   int32_t node[PS_CAP];
 };
 constexpr unsigned PFULL = 0xffffffffu;
+constexpr float SPLIT_ERR = 8e-15f;  // error of a hi/lo offset beyond FP32's relative one
+constexpr float H_SPLIT = 1e-8f;     // from here up a relative margin of 1e-5 covers it
 
 template <typename V>
 __device__ __forceinline__ V lanes_sum(V v) {
@@ -192,6 +201,8 @@ struct PseudoSolve {
   double rcut;
   float R = -1.f;  // radius the list covers (-1: none)
   int n = 0;       // its length; -1: it does not fit, every pass scans
+  bool sure = true;  // every density so far was within FP32's accuracy
+  bool alone = false;  // the last one was a tiny node's without neighbours: n = 1 / (pi h^3)
 
   // f(offset x, y, z, node, valid) over the candidates, 32 at a time, every lane calling
   template <typename F>
@@ -223,7 +234,7 @@ struct PseudoSolve {
 
   __device__ __forceinline__ void gather(float r) {
     const unsigned lt = (1u << lane) - 1u;
-    const float r2 = r * r * 1.00001f;
+    const float wide = (r + SPLIT_ERR) * 1.00001f, r2 = r >= 2.f * H_SPLIT ? r * r * 1.00001f : wide * wide;
     int c = 0;
     __syncwarp();
     scan([&](float x, float y, float z, int node, bool on) {
@@ -246,6 +257,9 @@ struct PseudoSolve {
   // n(h) and dn/dh, FP32
   __device__ __forceinline__ void density(float h, float& nn, float& dn) {
     cover(h);
+    // (the node itself lies at the offset 0 exactly)
+    alone = h < H_SPLIT && n == 1;
+    sure = sure && (h >= H_SPLIT || alone);
     const float ih = 1.0f / h;
     float s = 0.f, d = 0.f;
     auto add = [&](float x, float y, float z) {
@@ -270,10 +284,10 @@ struct PseudoSolve {
 
   // sums of w(q), q w'(q) and q^2 w''(q) + 2 q w'(q) at h, FP64 behind an FP32 screen
   __device__ __forceinline__ void sums64(double h, double& s, double& d, double& e) {
-    const float hf = (float)h, r2 = 4.00004f * hf * hf;
+    const float hf = (float)h, wide = 2.00001f * hf + SPLIT_ERR, r2 = hf >= H_SPLIT ? 4.00004f * hf * hf : wide * wide;
     cover(hf);
-    const double ih = 1.0 / h;
     s = d = e = 0.0;
+    const double ih = 1.0 / h;
     auto add = [&](int node) {
       const double* c = S.com + 3 * (int64_t)node;
       const double ex = (c[0] - px) * ih, ey = (c[1] - py) * ih, ez = (c[2] - pz) * ih;
@@ -299,13 +313,43 @@ struct PseudoSolve {
     d = lanes_sum(d);
     e = lanes_sum(e);
   }
+
+  // n(h) and dn/dh by FP64 sums
+  __device__ __forceinline__ void density64(double h, double& nn, double& dn) {
+    cover((float)h);
+    const double R2 = 4.0 * h * h, ih = 1.0 / h, norm = 1.0 / (MAP_PI * h * h * h);
+    double s = 0.0, d = 0.0;
+    auto add = [&](int node) {
+      const double* c = S.com + 3 * (int64_t)node;
+      const double dx = c[0] - px, dy = c[1] - py, dz = c[2] - pz;
+      const double r2 = dx * dx + dy * dy + dz * dz;
+      if (r2 >= R2) return;
+      const double q = sqrt(r2) * ih;
+      if (q < 1.0) {
+        const double w = 1.0 - 1.5 * q * q + 0.75 * q * q * q;
+        s += w;
+        d += 3.0 * w + q * (2.25 * q * q - 3.0 * q);
+      } else if (q < 2.0) {
+        const double t = 2.0 - q, w = 0.25 * t * t * t;
+        s += w;
+        d += 3.0 * w - 0.75 * t * t * q;
+      }
+    };
+    if (n >= 0)
+      for (int j = lane; j < n; j += 32) add(W.node[j]);
+    else
+      scan([&](float, float, float, int node, bool on) { if (on) add(node); });
+    nn = lanes_sum(s) * norm;
+    dn = -lanes_sum(d) * norm * ih;
+  }
 };
 
 // One warp per output slot holding an accepted node: Newton-Raphson on
 // h = hfact n(h)^(-1/3) from Eq. (9)'s guess, bisection on [h0/16, 16 h0]
 // when it fails, the guess itself when that has no sign change (Section
-// III-C); then Halley's step on sum_b w = pi hfact^3 in FP64.  The lanes hold
-// identical sums, so the iteration is warp-uniform.
+// III-C); then Halley's step on sum_b w = pi hfact^3 in FP64.  What FP32 cannot
+// decide is solved once more in FP64.  The lanes hold identical sums, so the
+// iteration is warp-uniform.
 __global__ void __launch_bounds__(PS_WARPS * 32) pseudo_h(int64_t nout, const int32_t* __restrict__ node_of_slot, NodeSet S,
                          const unsigned long long* __restrict__ size_bits, const int32_t* __restrict__ parent,
                          const int32_t* __restrict__ level, const int64_t* __restrict__ nb, const double* __restrict__ hs,
@@ -336,30 +380,36 @@ __global__ void __launch_bounds__(PS_WARPS * 32) pseudo_h(int64_t nout, const in
   const float hf_s = (float)hfact, hf_lo = (float)(hfact - (double)hf_s), hf3_s = (float)(hfact / 3.0);
   const double lo = g0 / 16.0, hi = g0 * 16.0;
   const float lo_s = (float)lo, hi_s = (float)hi;
+  // (of a node by itself: g = h (1 - hfact pi^(1/3)), and Newton's step is h)
+  const double g_alone = 1.0 - hfact * 1.4645918875615233;
   double h = g0;
-  bool ok = false, root = true;
+  bool ok = false, root = true, sure = true;
   float h32 = (float)g0;
   for (int it = 0; it < 30; ++it) {
     float nn, dn;
     P.density(h32, nn, dn);
+    if (P.alone && fabs(g_alone) > 1e-3) break;
     const float t = rcbrtf(nn);
     const float f = (h32 - hf_s * t) - hf_lo * t;
     const float fp = 1.f + hf3_s * (t * t) * (t * t) * dn;
     const float d = f / fp, hn = h32 - d;
-    if (!(hn >= lo_s && hn <= hi_s)) break;
+    sure = P.sure && it < 24 && clear_step(h32, d, fp, lo_s, hi_s);
+    if (!sure || !(hn >= lo_s && hn <= hi_s)) break;
     if (fabsf(hn - h32) < 1e-6f * hn) { h = (double)h32 - (double)d; ok = true; break; }
     h32 = hn;
   }
-  if (!ok) {
+  if (!ok && sure) {
     auto g = [&](double v) {
       float nn, dn;
       P.density((float)v, nn, dn);
-      return v - hfact * rcbrt((double)nn);
+      const double w = P.alone ? v * g_alone : v - hfact * rcbrt((double)nn);
+      sure = sure && P.sure && fabs(w) > 1e-4 * v;
+      return w;
     };
     if (!(g(lo) < 0.0 && g(hi) > 0.0)) {
       h = g0;
       root = false;
-    } else {
+    } else if (sure) {
       double a0 = lo, b0 = hi;
       for (int it = 0; it < 200; ++it) {
         const double mid = 0.5 * (a0 + b0);
@@ -367,19 +417,52 @@ __global__ void __launch_bounds__(PS_WARPS * 32) pseudo_h(int64_t nout, const in
         if (b0 - a0 < 1e-5 * mid) break;  // the FP64 steps below finish
       }
       h = 0.5 * (a0 + b0);
+      sure = P.sure;  // (a sign taken wrongly is one at the root)
     }
   }
-  if (root) {
+  if (root && sure) {
     // h <- h (1 + u), S' = -d/h, S'' = e/h^2; again while a step is so large that its cube shows
     const double target = MAP_PI * hfact * hfact * hfact;
+    sure = false;
     for (int it = 0; it < 30; ++it) {
       double s, d, e;
       P.sums64(h, s, d, e);
       const double F = s - target;
       const double u = 2.0 * F * d / (2.0 * d * d - F * e);
-      if (!(fabs(u) < 1e-2)) break;  // S' is 0 (no neighbour inside): the FP32 root stands
+      if (!(fabs(u) < 1e-2)) break;  // (no number where S' is 0)
       h += h * u;
-      if (fabs(u) < 2e-6) break;
+      if (fabs(u) < 2e-6) { sure = h > lo && h < hi; break; }
+    }
+  }
+  if (!sure) {
+    h = g0;
+    ok = false;
+    for (int it = 0; it < 30; ++it) {
+      double nn, dn;
+      P.density64(h, nn, dn);
+      const double t = rcbrt(nn), t2 = t * t;
+      const double hn = h - (h - hfact * t) / (1.0 + hfact / 3.0 * (t2 * t2 * dn));
+      if (!(hn >= lo && hn <= hi)) break;
+      ok = fabs(hn - h) < 1e-10 * hn;
+      h = hn;
+      if (ok) break;
+    }
+    if (!ok) {
+      auto g = [&](double v) {
+        double nn, dn;
+        P.density64(v, nn, dn);
+        return v - hfact * rcbrt(nn);
+      };
+      h = g0;
+      if (g(lo) < 0.0 && g(hi) > 0.0) {
+        double a0 = lo, b0 = hi;
+        for (int it = 0; it < 200; ++it) {
+          const double mid = 0.5 * (a0 + b0);
+          if (g(mid) < 0.0) a0 = mid; else b0 = mid;
+          if (b0 - a0 < 1e-12 * mid) break;
+        }
+        h = 0.5 * (a0 + b0);
+      }
     }
   }
   if (lane == 0) oh[j] = h;

@@ -108,3 +108,25 @@ def test_pseudo_mapping_reduces_pairs(cloud):
     assert rel_err(res["mass"], ref["mass"]).max() < 1e-5
     assert abs(res["mass"].sum() - ref["mass"].sum()) < 1e-7 * ref["mass"].sum()
     assert res["n_pairs"] < 0.5 * 100 * p.n
+
+
+@pytest.mark.parametrize("jitter", [1e-9, 1e-10, 1e-11, 1e-12])
+def test_tiny_nodes_keep_their_guess(jitter):
+    """A node of two particles that nearly coincide, far from all others, finds
+    no neighbour within 32 of its guesses: its h is Eq. (9)'s, 2 hfact s, to
+    the rounding of s (a few 1e-16)."""
+    r = np.random.default_rng(91)
+    base = r.random((2000, 3)) * 0.9 + 0.05
+    pos = np.concatenate([base, base + jitter * r.normal(size=base.shape)])
+    p = synth.Particles(*(np.ascontiguousarray(pos[:, k]) for k in range(3)), np.full(len(pos), 0.3 / len(pos)))
+    h, _ = oracle_h(p)
+    tiny = 0
+    for source in ([0.9, 0.8, 0.1], [0.1, 0.2, 0.9], [0.5, 0.5, 0.5]):
+        out = gpu_pseudo(p, h, source, theta=0.05)
+        for k in np.nonzero(out["kind"] == 0)[0]:
+            d = np.linalg.norm(pos - [out["x"][k], out["y"][k], out["z"][k]], axis=1)
+            near = d < 100 * jitter
+            if near.sum() == 2 and abs(out["m"][k] / (2 * p.m[0]) - 1) < 1e-9:
+                tiny += 1
+                assert abs(out["h"][k] / (2 * oracle.HFACT * d[near].max()) - 1) < 1e-12
+    assert tiny > 10
