@@ -585,13 +585,6 @@ __device__ __forceinline__ bool bracket_root(double g0, double lo, double hi, G 
   return y > lo || g(lo) < 0.0;
 }
 
-// A step of FP32's Newton that FP64's would not take otherwise: the slope is
-// neither flat nor out of range, and the new iterate lies clear of the bounds.
-__device__ __forceinline__ bool clear_step(float fp, float hn, float lo, float hi) {
-  return fabsf(fp) > 0.02f && fabsf(fp) < 50.f &&
-         ((hn > 1.001f * lo && hn < 0.999f * hi) || hn < 0.999f * lo || hn > 1.001f * hi);
-}
-
 // redo, n_redo (FP64 build): the positions left to h_solve_exact.
 template <bool MIXED, int LONG>
 __global__ void __launch_bounds__(HS_WARPS * 32)
@@ -648,7 +641,7 @@ __global__ void __launch_bounds__(HS_WARPS * 32)
         const float d = f / fp;
         const float hn = hs - d;
         if (!MIXED) {
-          sure = it < 24 && clear_step(fp, hn, lo_s, hi_s);
+          sure = it < 24 && clear_step(hs, d, fp, lo_s, hi_s);
           if (!sure) break;
         }
         if (!(hn >= lo_s && hn <= hi_s)) break;
