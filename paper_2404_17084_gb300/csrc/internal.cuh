@@ -352,6 +352,8 @@ int tree_build(map_ctx* ctx, const double* x, const double* y, const double* z, 
 // particles, tree_nodes_max(n, leaf).  Same nodes, same order, same sums as
 // tree_build.
 int64_t tree_nodes_max(int64_t n, int leaf_size);
+// entries of the scan a tree build takes its node numbers from
+int64_t tree_scan_entries(int64_t n);
 int tree_build_graph(map_ctx* ctx, const double* x, const double* y, const double* z, const double* m,
                      const double* h, int64_t n, cudaStream_t s);
 // Output buffers of a pair-list build; nullptr members mean the context's

@@ -67,7 +67,7 @@ int setup_device(int dev) {
   S.base = static_cast<unsigned char*>(p);
   map_ctx& C = S.ctx;
   map_config_default(&C.cfg);
-  C.cfg.precision = MAP_FP64;  // the FP64 Newton tolerance, as solve_h on an FP64 context
+  C.cfg.precision = MAP_FP64;  // FP64's h and routes, as solve_h on an FP64 context
   C.cfg.device = dev;
   C.device = dev;
   if (cudaDeviceGetAttribute(&C.sm_count, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) return MAP_ECUDA;
@@ -83,17 +83,15 @@ int setup_device(int dev) {
   const size_t N = (size_t)NOALLOC_MAX_N, slack = 512;
   const size_t NC = 2 * N;  // node capacity
   bool ok = true;
-  ok &= take(C.ws_tree[0], 8 * N + slack);   // Morton keys (unsorted)
-  ok &= take(C.ws_tree[1], 4 * N + slack);   // indices (unsorted)
+  ok &= take(C.ws_tree[0], 8 * N + slack);   // Morton keys (unsorted), then the node maps
+  ok &= take(C.ws_tree[1], 4 * N + slack);   // indices (unsorted), then the maps' scan
   ok &= take(C.ws_tree[2], 8 * N + slack);   // sorted keys
   ok &= take(C.ws_tree[3], 4 * N + slack);   // sorted indices
   ok &= take(C.ws_tree[4], 40 * N + slack);  // sorted x, y, z, m, h
   ok &= take(C.ws_tree[5], 4 * N + slack);   // leaf of each sorted position
-  ok &= take(C.ws_tree[6], 4 * (NC + 1) + slack);
-  ok &= take(C.ws_tree[7], 8 * (NC + 1) + slack);
   const size_t esz[12] = {8, 4, 8, 8, 8, 4, 4, 8, 24, 8, 8, 48};
-  for (int k = 0; k < 12; ++k) ok &= take(C.ws_tree[8 + k], esz[k] * NC);
-  ok &= take(C.ws_tree[20], 24 * NC + slack);
+  for (int k = 0; k < 12; ++k) ok &= take(C.ws_tree[8 + k], esz[k] * NC + slack);
+  ok &= take(C.ws_tree[20], 24 * NC + slack);  // sums of m x
   ok &= take(C.ws_tree[21], 4 * NC + slack);
   ok &= take(C.ws_tree[22], 8 * N + slack);
   ok &= take(C.ws_tree[23], 24 * N + slack);  // FP32 hi/lo split coordinates
@@ -106,7 +104,7 @@ int setup_device(int dev) {
   size_t rs = 0, sc = 0;
   if (cub::DeviceRadixSort::SortPairs(nullptr, rs, (uint64_t*)nullptr, (uint64_t*)nullptr, (int32_t*)nullptr,
                                       (int32_t*)nullptr, (int64_t)N, 0, 63) != cudaSuccess ||
-      cub::DeviceScan::ExclusiveSum(nullptr, sc, (int32_t*)nullptr, (int64_t*)nullptr, (int64_t)(NC + 1)) !=
+      cub::DeviceScan::ExclusiveSum(nullptr, sc, (int32_t*)nullptr, (int32_t*)nullptr, tree_scan_entries((int64_t)N)) !=
           cudaSuccess)
     return MAP_ECUDA;
   const size_t need = (rs > sc ? rs : sc) + 4096;
@@ -120,7 +118,7 @@ int setup_device(int dev) {
   C.tree.level_begin.reserve(64);
   // the node arrays take their whole slots from the start, so that a tree
   // never needs to grow them (growth would be refused): any tree of up to NC
-  // nodes fits, whatever the order in which its levels fill
+  // nodes fits
   C.node_cap0 = (int64_t)NC;
   S.ready = true;
   return MAP_OK;

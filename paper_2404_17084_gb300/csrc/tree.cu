@@ -415,40 +415,27 @@ __global__ void level_starts(int64_t nw, const int32_t* __restrict__ base, int64
 
 // ---------------------------------------------------------------- tree build
 
-static int grow_nodes(map_ctx* ctx, int64_t need) {
+// The node arrays, for at least need nodes (nothing in them outlives a build).
+static int ensure_nodes(map_ctx* ctx, int64_t need) {
   DevTree& T = ctx->tree;
-  // node arrays live in ws_tree[8..19]; growing keeps the old contents
-  struct Arr { int slot; size_t esz; void** p; };
-  Arr arrs[] = {{8, sizeof(int64_t), (void**)&T.label},      {9, sizeof(int32_t), (void**)&T.level},
-                {10, sizeof(int64_t), (void**)&T.begin},     {11, sizeof(int64_t), (void**)&T.end},
-                {12, sizeof(int64_t), (void**)&T.first_child}, {13, sizeof(int32_t), (void**)&T.nchild},
-                {14, sizeof(int32_t), (void**)&T.parent},    {15, sizeof(double), (void**)&T.mass},
-                {16, 3 * sizeof(double), (void**)&T.com},    {17, sizeof(unsigned long long), (void**)&T.size_bits},
-                {18, sizeof(unsigned long long), (void**)&T.hmax_bits},
-                {19, 6 * sizeof(unsigned long long), (void**)&T.bbox_bits}};
-  for (auto& a : arrs) {
-    DevBuf& b = ctx->ws_tree[a.slot];
-    size_t bytes = (size_t)need * a.esz;
-    if (b.cap >= bytes) { *a.p = b.p; continue; }
-    size_t nb = bytes + bytes / 2 + 4096;
-    if (ctx->cfg.hbm_budget && ctx->bytes_in_use + nb > ctx->cfg.hbm_budget) return MAP_ENOMEM;
-    void* np = nullptr;
-    MAP_TRY(dev_alloc(ctx, &np, nb));
-    ctx->bytes_in_use += nb;
-    if (b.p) {
-      CUDA_TRY(cudaMemcpyAsync(np, b.p, b.cap, cudaMemcpyDeviceToDevice, ctx->cur_stream));
-      dev_free(ctx, b.p);
-      ctx->bytes_in_use -= b.cap;
-    }
-    b.p = np;
-    b.cap = nb;
-    *a.p = np;
-  }
+  MAP_TRY(ensure_t(ctx, ctx->ws_tree[8], need, &T.label));
+  MAP_TRY(ensure_t(ctx, ctx->ws_tree[9], need, &T.level));
+  MAP_TRY(ensure_t(ctx, ctx->ws_tree[10], need, &T.begin));
+  MAP_TRY(ensure_t(ctx, ctx->ws_tree[11], need, &T.end));
+  MAP_TRY(ensure_t(ctx, ctx->ws_tree[12], need, &T.first_child));
+  MAP_TRY(ensure_t(ctx, ctx->ws_tree[13], need, &T.nchild));
+  MAP_TRY(ensure_t(ctx, ctx->ws_tree[14], need, &T.parent));
+  MAP_TRY(ensure_t(ctx, ctx->ws_tree[15], need, &T.mass));
+  MAP_TRY(ensure_t(ctx, ctx->ws_tree[16], 3 * need, &T.com));
+  MAP_TRY(ensure_t(ctx, ctx->ws_tree[17], need, &T.size_bits));
+  MAP_TRY(ensure_t(ctx, ctx->ws_tree[18], need, &T.hmax_bits));
+  MAP_TRY(ensure_t(ctx, ctx->ws_tree[19], 6 * need, &T.bbox_bits));
   return MAP_OK;
 }
 
-// The sorted particles and, in ws_tree[6] and [7], the node maps and their
-// scan; *total: the node count on the device.
+// The sorted particles, and the node maps and their scan in the buffers of the
+// unsorted keys (maps and counts, 5.5 of 8 bytes per particle) and indices (the
+// scan, 2.75 of 4), which are done with then.
 static int tree_nodes(map_ctx* ctx, const double* x, const double* y, const double* z, const double* m, const double* h,
                       int64_t n, cudaStream_t s, uint32_t** map, int32_t** base) {
   DevTree& T = ctx->tree;
@@ -456,8 +443,9 @@ static int tree_nodes(map_ctx* ctx, const double* x, const double* y, const doub
   const int tpb = 256;
   uint64_t* keys_in;
   int32_t* idx_in;
-  MAP_TRY(ensure_t(ctx, ctx->ws_tree[0], n, &keys_in));
-  MAP_TRY(ensure_t(ctx, ctx->ws_tree[1], n, &idx_in));
+  const int64_t nw = (n + 31) / 32, entries = LEVELS * nw, room = n > entries + 1 ? n : entries + 1;
+  MAP_TRY(ensure_t(ctx, ctx->ws_tree[0], room, &keys_in));
+  MAP_TRY(ensure_t(ctx, ctx->ws_tree[1], room, &idx_in));
   MAP_TRY(ensure_t(ctx, ctx->ws_tree[2], n, &T.keys));
   MAP_TRY(ensure_t(ctx, ctx->ws_tree[3], n, &T.idx));
   MAP_TRY(ensure_t(ctx, ctx->ws_tree[4], 5 * n, &T.xs));
@@ -482,11 +470,9 @@ static int tree_nodes(map_ctx* ctx, const double* x, const double* y, const doub
   gather_sorted<<<nblk(n, tpb), tpb, 0, s>>>(n, T.idx, x, y, z, m, h, T.xs, T.ys, T.zs, T.ms, T.hs, T.split,
                                              T.hs32); ++ctx->launches;
   CUDA_TRY(cudaGetLastError());
-  const int64_t nw = (n + 31) / 32, entries = LEVELS * nw;
-  int32_t* count;
-  MAP_TRY(ensure_t(ctx, ctx->ws_tree[6], 2 * entries + 1, map));
-  count = reinterpret_cast<int32_t*>(*map + entries);
-  MAP_TRY(ensure_t(ctx, ctx->ws_tree[7], entries + 1, base));
+  *map = reinterpret_cast<uint32_t*>(keys_in);
+  int32_t* count = reinterpret_cast<int32_t*>(*map + entries);
+  *base = idx_in;
   tree_bits<<<nblk(nw * 32, tpb), tpb, 0, s>>>(n, nw, T.keys, ctx->cfg.leaf_size, *map, count); ++ctx->launches;
   CUDA_TRY(cudaGetLastError());
   size_t sb = 0;
@@ -504,7 +490,7 @@ static int tree_records(map_ctx* ctx, int64_t n, int64_t cap, const uint32_t* ma
   double* msum;
   int32_t* arrived;
   float* box32;
-  MAP_TRY(ensure_t(ctx, ctx->ws_tree[20], 3 * cap, &msum));
+  MAP_TRY(ensure_t(ctx, ctx->ws_tree[20], 3 * cap + LEVELS + 1, &msum));
   MAP_TRY(ensure_t(ctx, ctx->ws_tree[21], cap, &arrived));
   MAP_TRY(ensure_t(ctx, ctx->ws_tree[24], 8 * cap, &box32));
   T.box32 = box32;
@@ -533,23 +519,19 @@ int tree_build(map_ctx* ctx, const double* x, const double* y, const double* z, 
   // fixed-workspace context has from the start
   int64_t cap = n / 4 + 64;
   if (ctx->node_cap0 > cap) cap = ctx->node_cap0;
-  MAP_TRY(grow_nodes(ctx, cap));
+  MAP_TRY(ensure_nodes(ctx, cap));
   int32_t* total = reinterpret_cast<int32_t*>(ctx->h_scratch);
   CUDA_TRY(cudaMemcpyAsync(total, base + LEVELS * nw, sizeof(int32_t), cudaMemcpyDeviceToHost, s));
   CUDA_TRY(cudaStreamSynchronize(s));
   T.nnodes = *total;
-  if (T.nnodes > cap) {
-    cap = T.nnodes + T.nnodes / 8;
-    MAP_TRY(grow_nodes(ctx, cap));
-  }
+  if (T.nnodes > cap) MAP_TRY(ensure_nodes(ctx, T.nnodes));
   T.level_begin.clear();
   MAP_TRY(tree_records(ctx, n, T.nnodes, map, base, s));
   if (want_size) {
-    // the walk also needs the levels' first nodes, and the node sizes
-    // (in the buffers of the unsorted indices and keys, which are done with)
-    int64_t* starts = reinterpret_cast<int64_t*>(ctx->ws_tree[1].p);
+    // the walk also needs the levels' first nodes (in the place of the sums of m
+    // x) and the node sizes (the slices' list in the maps' place): both done with
+    int64_t* starts = reinterpret_cast<int64_t*>(ctx->ws_tree[20].p);
     int64_t* big = reinterpret_cast<int64_t*>(ctx->ws_tree[0].p);
-    if (ctx->ws_tree[1].cap < (LEVELS + 1) * sizeof(int64_t)) return MAP_EINVAL;  // (never: 256 bytes at least)
     level_starts<<<1, 32, 0, s>>>(nw, base, starts); ++ctx->launches;
     CUDA_TRY(cudaGetLastError());
     T.level_begin.resize(LEVELS + 1);
@@ -571,6 +553,8 @@ int tree_build(map_ctx* ctx, const double* x, const double* y, const double* z, 
   return MAP_OK;
 }
 
+int64_t tree_scan_entries(int64_t n) { return LEVELS * ((n + 31) / 32) + 1; }
+
 // ---------------------------------------------------------------- tree build with no host reads
 
 int64_t tree_nodes_max(int64_t n, int leaf_size) {
@@ -588,7 +572,7 @@ int tree_build_graph(map_ctx* ctx, const double* x, const double* y, const doubl
   int32_t* base;
   MAP_TRY(tree_nodes(ctx, x, y, z, m, h, n, s, &map, &base));
   const int64_t cap = tree_nodes_max(n, ctx->cfg.leaf_size);
-  MAP_TRY(grow_nodes(ctx, cap));
+  MAP_TRY(ensure_nodes(ctx, cap));
   MAP_TRY(tree_records(ctx, n, cap, map, base, s));
   // host-side sizes are unknown without a read: an upper bound, no levels
   T.nnodes = cap;

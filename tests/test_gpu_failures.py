@@ -113,3 +113,51 @@ def test_budget_below_one_request(small):
         assert rel_err(mass.cpu().numpy(), ref["mass"]).max() < 1e-5
     finally:
         L.map_destroy(ctx)
+
+
+# call, particles, particles per cell, precision (0 FP64, 1 mixed) and an
+# hbm_budget in MiB that holds it: half a percent above the least of the
+# library's first level-by-level octree and two-pass walk
+BUDGETS = [("solve_h", 2000, 1, 1, 0.489), ("pseudo", 2000, 1, 1, 0.581), ("solve_h", 60013, 1, 0, 12.34),
+           ("pseudo", 60013, 1, 1, 14.16)]
+
+
+@pytest.mark.parametrize("call,n,per_cell,precision,mib", BUDGETS)
+def test_budgets_that_held_a_call_still_do(call, n, per_cell, precision, mib):
+    """Workspaces shrink, or are given up for slower forms, before a call is
+    refused; the result is the one without a budget, bit for bit."""
+    L = lib()
+    p = synth.lognormal_particles(n, 3 if n < 10000 else 4, ngrid=64)
+    x, y, z, m, h = dev_particles(p)
+    out = []
+    for budget in (0, int(mib * 2 ** 20)):
+        ctx = L.map_init(L.map_config_default(precision=precision, hbm_budget=budget))
+        try:
+            if call == "solve_h":
+                L.solve_h(ctx, L.make_particles(x, y, z, None, h))
+                out.append([h.clone()])
+            elif call == "pseudo":
+                o = [torch.zeros(n, dtype=torch.float64, device="cuda") for _ in range(5)]
+                L.build_pseudo_particles(ctx, L.make_particles(x, y, z, m, torch.full_like(x, 0.03)), [0.5, 0.5, 0.5],
+                                         L.make_particles(*o))
+                out.append(o)
+            elif call == "grid":
+                g, _ = L.map_grid_build(ctx, x, y, z, lloyd=1, merge_tol=1e-9)
+                out.append(list(L.map_grid_copy(ctx, g).values()))
+            else:
+                keep = np.sort(np.random.default_rng(9).choice(n, n // per_cell, replace=False))
+                grid = synth.voronoi(p.pos()[keep])
+                if not out:
+                    hctx = L.map_init(L.map_config_default(precision=1))
+                    L.solve_h(hctx, L.make_particles(x, y, z, None, h))
+                    L.map_destroy(hctx)
+                hd = L.map_grid_upload(ctx, L.grid_to_device(grid))
+                mass = torch.empty(grid.ncell, dtype=torch.float64, device="cuda")
+                L.map_particles_to_cells(ctx, L.make_particles(x, y, z, m, h), hd, mass)
+                out.append([mass])
+                if call == "inverse":
+                    out[-1].append(L.map_cells_to_particles(ctx, torch.ones_like(mass), torch.empty_like(x)))
+        finally:
+            L.map_destroy(ctx)
+    for a, b in zip(*out):
+        assert torch.equal(a, b)
