@@ -73,6 +73,14 @@ void dev_free(map_ctx* ctx, void* p) {
 int ctx_ensure(map_ctx* ctx, DevBuf& b, size_t bytes) {
   if (b.cap >= bytes) return MAP_OK;
   size_t nb = bytes + bytes / 4 + 4096;
+  // over the budget: the pair walk's rows go first, when the list is made
+  DevBuf& rows = ctx->ws_pairs[8];
+  if (ctx->cfg.hbm_budget && ctx->bytes_in_use - b.cap + nb > ctx->cfg.hbm_budget && ctx->rows_done && rows.p &&
+      &b != &rows) {
+    dev_free(ctx, rows.p);
+    ctx->bytes_in_use -= rows.cap;
+    rows = DevBuf();
+  }
   size_t after = ctx->bytes_in_use - b.cap + nb;
   if (ctx->cfg.hbm_budget && after > ctx->cfg.hbm_budget) return MAP_ENOMEM;
   if (b.p) {

@@ -163,6 +163,7 @@ struct map_ctx {
   DevBuf ws_vor[23];                   // grid construction: buckets, cell slots, CSR arrays
   DevBuf ws_inv[15];                   // particle-major copy of the pair list (inverse mapping, Eq. 4)
   DevBuf cub_tmp;
+  bool rows_done = false;              // ws_pairs[8], the pair walk's rows, holds nothing a later step reads
   DevTree tree;
   int64_t node_cap0 = 0;  // > 0: octree node arrays start at this capacity (a context whose workspace is fixed)
   int item_target = 16;   // work items per resident warp of the integral launch (the autotuner may raise it)

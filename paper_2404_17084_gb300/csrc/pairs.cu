@@ -705,8 +705,9 @@ struct PairWalk {
 };
 
 // Every cell's pairs in its row (or on the list of cells to walk again), and
-// their counts.
-int walk_rows(map_ctx* ctx, const PreparedGrid* g, cudaStream_t s, PairWalk& P) {
+// their counts.  pool = false: rows without a pool, for a budget that holds no
+// more (every cell past its row is walked again).
+int walk_rows(map_ctx* ctx, const PreparedGrid* g, cudaStream_t s, PairWalk& P, bool pool) {
   DevTree& T = ctx->tree;
   const int64_t nc = g->ncell;
   const int tpb = 128;
@@ -728,10 +729,11 @@ int walk_rows(map_ctx* ctx, const PreparedGrid* g, cudaStream_t s, PairWalk& P) 
                  T.hmax_bits, T.box32};
   P.G = PairGrid{g->cell_face_off, g->face_plane, g->face32, g->site, g->rad, g->rin};
   MAP_TRY(ensure_t(ctx, ctx->ws_pairs[0], nc + 1, &P.count));
-  const int64_t npool = nc / 32 + (2 * nc < 4096 ? 2 * nc : 4096);
+  const int64_t npool = pool ? nc / 32 + (2 * nc < 4096 ? 2 * nc : 4096) : 0;
   int32_t* buf;
-  MAP_TRY(ensure_t(ctx, ctx->ws_pairs[8], (size_t)(nc + npool) * (PAIR_ROW + 1), &buf));
+  ctx->rows_done = false;
   MAP_TRY(ensure_t(ctx, ctx->ws_pairs[9], nc, &P.Q.again));
+  MAP_TRY(ensure_t(ctx, ctx->ws_pairs[8], (size_t)(nc + npool) * (PAIR_ROW + 1), &buf));
   P.Q.rows = buf;
   P.Q.pool = buf + nc * PAIR_ROW;
   P.Q.first = P.Q.pool + npool * PAIR_ROW;
@@ -774,30 +776,55 @@ int walk_list(map_ctx* ctx, const PairWalk& P, int64_t nc, const int64_t* off, i
                                                                                list, cap);
   ++ctx->launches;
   CUDA_TRY(cudaGetLastError());
+  ctx->rows_done = true;
   return MAP_OK;
+}
+
+// The walk, the list's offsets and the list (np < 0: its length is read back,
+// else np is its room).
+int walk_to_list(map_ctx* ctx, const PreparedGrid* g, cudaStream_t s, const PairBufs& out, bool pool, int64_t& np,
+                 int64_t** off, int32_t** list) {
+  const int64_t nc = g->ncell;
+  PairWalk P;
+  MAP_TRY(walk_rows(ctx, g, s, P, pool));
+  MAP_TRY(ensure_t(ctx, out.off ? *out.off : ctx->ws_pairs[1], nc + 1, off));
+  size_t tb = 0;
+  CUDA_TRY(cub::DeviceScan::ExclusiveSum(nullptr, tb, P.count, *off, nc + 1, s));
+  MAP_TRY(ctx_ensure(ctx, ctx->cub_tmp, tb));
+  CUDA_TRY(cub::DeviceScan::ExclusiveSum(ctx->cub_tmp.p, tb, P.count, *off, nc + 1, s));
+  const bool read = np < 0;
+  if (read) {
+    CUDA_TRY(cudaMemcpyAsync(ctx->h_scratch, *off + nc, sizeof(int64_t), cudaMemcpyDeviceToHost, s));
+    CUDA_TRY(cudaStreamSynchronize(s));
+    np = ctx->h_scratch[0];
+  }
+  MAP_TRY(ensure_t(ctx, out.idx ? *out.idx : ctx->ws_pairs[3], np + 1, list));
+  return walk_list(ctx, P, nc, *off, *list, read ? INT64_MAX : np, s);
+}
+
+// The same, without the pool when the budget does not hold it.
+int build_list(map_ctx* ctx, const PreparedGrid* g, cudaStream_t s, const PairBufs& out, int64_t& np, int64_t** off,
+               int32_t** list) {
+  const int64_t np0 = np;
+  const int r = walk_to_list(ctx, g, s, out, true, np, off, list);
+  if (r != MAP_ENOMEM) return r;
+  DevBuf& rows = ctx->ws_pairs[8];
+  dev_free(ctx, rows.p);
+  ctx->bytes_in_use -= rows.cap;
+  rows = DevBuf();
+  np = np0;
+  return walk_to_list(ctx, g, s, out, false, np, off, list);
 }
 
 }  // namespace
 
 int pairs_build(map_ctx* ctx, const PreparedGrid* g, cudaStream_t s, const PairBufs& out) {
   const int64_t nc = g->ncell;
-  PairWalk P;
-  MAP_TRY(walk_rows(ctx, g, s, P));
-  int64_t* count = P.count;
-  int64_t* off;
-  MAP_TRY(ensure_t(ctx, out.off ? *out.off : ctx->ws_pairs[1], nc + 1, &off));
-  size_t tb = 0;
-  CUDA_TRY(cub::DeviceScan::ExclusiveSum(nullptr, tb, count, off, nc + 1, s));
-  MAP_TRY(ctx_ensure(ctx, ctx->cub_tmp, tb));
-  CUDA_TRY(cub::DeviceScan::ExclusiveSum(ctx->cub_tmp.p, tb, count, off, nc + 1, s));
-  CUDA_TRY(cudaMemcpyAsync(ctx->h_scratch, off + nc, sizeof(int64_t), cudaMemcpyDeviceToHost, s));
-  CUDA_TRY(cudaStreamSynchronize(s));
-  const int64_t np = ctx->h_scratch[0];
   // the list in the walk's order (deterministic); map_get_pairs and
   // map_copy_pairs sort each cell's entries by particle index when read
+  int64_t np = -1, *off;
   int32_t* list;
-  MAP_TRY(ensure_t(ctx, out.idx ? *out.idx : ctx->ws_pairs[3], np + 1, &list));
-  MAP_TRY(walk_list(ctx, P, nc, off, list, INT64_MAX, s));
+  MAP_TRY(build_list(ctx, g, s, out, np, &off, &list));
   ctx->n_pairs = np;
   ctx->pair_off = off;
   ctx->pair_idx = list;
@@ -847,18 +874,9 @@ int pairs_build_graph(map_ctx* ctx, const PreparedGrid* g, cudaStream_t s, const
                       int64_t cap_items) {
   if (!out.off || !out.idx || !out.items || !out.ioff || !out.part) return MAP_EINVAL;
   const int64_t nc = g->ncell;
-  PairWalk P;
-  MAP_TRY(walk_rows(ctx, g, s, P));
-  int64_t* count = P.count;
-  int64_t* off;
-  MAP_TRY(ensure_t(ctx, *out.off, nc + 1, &off));
-  size_t tb = 0;
-  CUDA_TRY(cub::DeviceScan::ExclusiveSum(nullptr, tb, count, off, nc + 1, s));
-  MAP_TRY(ctx_ensure(ctx, ctx->cub_tmp, tb));
-  CUDA_TRY(cub::DeviceScan::ExclusiveSum(ctx->cub_tmp.p, tb, count, off, nc + 1, s));
+  int64_t np = cap_pairs, *off;
   int32_t* list;
-  MAP_TRY(ensure_t(ctx, *out.idx, cap_pairs + 1, &list));
-  MAP_TRY(walk_list(ctx, P, nc, off, list, cap_pairs, s));
+  MAP_TRY(build_list(ctx, g, s, out, np, &off, &list));
   // the work items (the item size from the device-side pair count)
   const int64_t tgt = (int64_t)ctx->item_target * ctx->sm_count * 24;
   int64_t *icnt, *ioff;
@@ -867,7 +885,7 @@ int pairs_build_graph(map_ctx* ctx, const PreparedGrid* g, cudaStream_t s, const
   item_count<<<nblk(nc, 256), 256, 0, s>>>(nc, off, tgt, icnt); ++ctx->launches;
   CUDA_TRY(cudaGetLastError());
   CUDA_TRY(cudaMemsetAsync(icnt + nc, 0, sizeof(int64_t), s));
-  tb = 0;
+  size_t tb = 0;
   CUDA_TRY(cub::DeviceScan::ExclusiveSum(nullptr, tb, icnt, ioff, nc + 1, s));
   MAP_TRY(ctx_ensure(ctx, ctx->cub_tmp, tb));
   CUDA_TRY(cub::DeviceScan::ExclusiveSum(ctx->cub_tmp.p, tb, icnt, ioff, nc + 1, s));

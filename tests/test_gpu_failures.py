@@ -118,7 +118,8 @@ def test_budget_below_one_request(small):
 # call, particles, particles per cell, precision (0 FP64, 1 mixed) and an
 # hbm_budget in MiB that holds it: half a percent above the least of the
 # library's first level-by-level octree and two-pass walk
-BUDGETS = [("solve_h", 2000, 1, 1, 0.489), ("pseudo", 2000, 1, 1, 0.581), ("solve_h", 60013, 1, 0, 12.34),
+BUDGETS = [("solve_h", 2000, 1, 1, 0.489), ("map", 2000, 1, 1, 19.08), ("map", 2000, 1, 0, 24.39),
+           ("pseudo", 2000, 1, 1, 0.581), ("solve_h", 60013, 1, 0, 12.34), ("map", 60013, 30, 1, 38.12),
            ("pseudo", 60013, 1, 1, 14.16)]
 
 
