@@ -187,6 +187,7 @@ struct map_ctx {
   const int32_t* inv_order = nullptr; // places on the particles' curve in the order of the work
   const int32_t* inv_pid = nullptr;   // the particle at each place
   const int64_t* inv_nlong = nullptr; // device: particles summed by a whole warp
+  int64_t inv_longest = 0;            // at most that many
   struct PairItem* items = nullptr;  // work items of the pair-integral kernel
   int64_t* item_off = nullptr;       // [ncell+1]: items of cell c
   double* partial = nullptr;         // per item: its pairs' mass

@@ -92,15 +92,16 @@ __global__ void inv_bounds(int64_t np, int64_t n, const int32_t* __restrict__ ke
 constexpr unsigned INV_LONG = 256;
 constexpr int INV_WINDOW = 10;
 
-// (nlong, zeroed: the number of long particles)
-__global__ void inv_keys(int64_t n, const int64_t* __restrict__ ioff, uint32_t* __restrict__ key,
+// (long_above: INV_LONG, or 0 when every particle with entries is long; nlong,
+// zeroed: the number of long particles)
+__global__ void inv_keys(int64_t n, int64_t long_above, const int64_t* __restrict__ ioff, uint32_t* __restrict__ key,
                          int32_t* __restrict__ ids, unsigned long long* nlong) {
   const int64_t stride = (int64_t)gridDim.x * blockDim.x;
   for (int64_t a = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; a < n; a += stride) {
     const int64_t c = ioff[a + 1] - ioff[a];
-    key[a] = c > INV_LONG ? 0u : (uint32_t)(((a >> INV_WINDOW) + 1) << 9 | (int64_t)(INV_LONG - c));
+    key[a] = c > long_above ? 0u : (uint32_t)(((a >> INV_WINDOW) + 1) << 9 | (int64_t)(INV_LONG - c));
     ids[a] = (int32_t)a;
-    const unsigned here = __activemask(), m = __ballot_sync(here, c > INV_LONG);
+    const unsigned here = __activemask(), m = __ballot_sync(here, c > long_above);
     if (m && (int)(threadIdx.x & 31) == __ffs(here) - 1) atomicAdd(nlong, (unsigned long long)__popc(m));
   }
 }
@@ -237,7 +238,9 @@ int bits_for(int64_t n) {
   return b;
 }
 
-int build_index(map_ctx* ctx, cudaStream_t s) {
+// groups = false: every particle's entries contiguous, summed by a warp of its
+// own, for a budget that does not hold the groups' padding.
+int build_index(map_ctx* ctx, cudaStream_t s, bool groups) {
   const int64_t np = ctx->n_pairs, nc = ctx->last_ncell, n = ctx->last_npart;
   int64_t* ioff;
   MAP_TRY(ensure_t(ctx, ctx->ws_inv[0], n + 1, &ioff));
@@ -253,7 +256,9 @@ int build_index(map_ctx* ctx, cudaStream_t s) {
   // largest - its smallest count), the group that crosses into the next window
   // by 32 x 256, the last one by its missing lanes: 16 entries per particle and
   // 3 x 8192 hold them all.
-  const int64_t room = np + 16 * n + 3 * 8192;
+  const int64_t room = groups ? np + 16 * n + 3 * 8192 : np;
+  // (the particles of more than INV_LONG entries: at most np / (INV_LONG + 1))
+  const int64_t longest = groups && np / (INV_LONG + 1) < n ? np / (INV_LONG + 1) : n;
   unsigned long long* val_s = nullptr;
   if (np > 0) {
     unsigned long long* val;  // (in the place of f_ai, and key in the cells' place, which are written after the sort)
@@ -288,13 +293,14 @@ int build_index(map_ctx* ctx, cudaStream_t s) {
   uint32_t *okey, *okey_s;
   int32_t *ids, *order;
   MAP_TRY(ensure_t(ctx, ctx->ws_inv[7], 2 * n, &okey));
-  MAP_TRY(ensure_t(ctx, ctx->ws_inv[8], n, &ids));
+  ids = place;  // (done with)
   MAP_TRY(ensure_t(ctx, ctx->ws_inv[9], n, &order));
   okey_s = okey + n;
   int64_t* nlong;
   MAP_TRY(ensure_t(ctx, ctx->ws_inv[10], 1, &nlong));
   CUDA_TRY(cudaMemsetAsync(nlong, 0, sizeof(int64_t), s));
-  inv_keys<<<g, 256, 0, s>>>(n, ioff, okey, ids, reinterpret_cast<unsigned long long*>(nlong)); ++ctx->launches;
+  inv_keys<<<g, 256, 0, s>>>(n, groups ? INV_LONG : 0, ioff, okey, ids, reinterpret_cast<unsigned long long*>(nlong));
+  ++ctx->launches;
   CUDA_TRY(cudaGetLastError());
   size_t tb2 = 0;
   const int cb = bits_for(((n >> INV_WINDOW) + 2) << 9);
@@ -321,6 +327,9 @@ int build_index(map_ctx* ctx, cudaStream_t s) {
   }
   ctx->inv_order = order;
   ctx->inv_nlong = nlong;
+  ctx->inv_longest = longest;
+  double* cv;  // (the call's cell values, so that a call after this one finds its room)
+  MAP_TRY(ensure_t(ctx, ctx->ws_inv[12], nc, &cv));
   ctx->inv_ready = true;
   // the copy reads the pair list, which a later map_get_pairs sorts in place:
   // that sort runs on this call's stream or one ordered after it (ctx_enter)
@@ -337,7 +346,19 @@ extern "C" int map_cells_to_particles(map_ctx* ctx, const double* cell_value, do
   if (n == 0) return MAP_OK;
   cudaStream_t s = reinterpret_cast<cudaStream_t>(stream);
   MAP_ENTER(ctx, s);
-  if (!ctx->inv_ready) MAP_TRY(build_index(ctx, s));
+  if (!ctx->inv_ready) {
+    int r = build_index(ctx, s, true);
+    if (r == MAP_ENOMEM) {
+      for (int k : {1, 2, 14}) {
+        DevBuf& b = ctx->ws_inv[k];
+        dev_free(ctx, b.p);
+        ctx->bytes_in_use -= b.cap;
+        b = DevBuf();
+      }
+      r = build_index(ctx, s, false);
+    }
+    if (r != MAP_OK) return r;
+  }
   if (!ctx->inv_cell) {  // no pairs: every sum is empty
     CUDA_TRY(cudaMemsetAsync(particle_value, 0, n * sizeof(double), s));
     return MAP_OK;
@@ -347,10 +368,9 @@ extern "C" int map_cells_to_particles(map_ctx* ctx, const double* cell_value, do
   MAP_TRY(ensure_t(ctx, ctx->ws_inv[12], nc, &cv));
   inv_permute<<<(unsigned)ctx->sm_count * 8, 256, 0, s>>>(nc, ctx->inv_morton, cell_value, cv); ++ctx->launches;
   CUDA_TRY(cudaGetLastError());
-  // a warp per item; their number, at most a long particle each for the first
-  // np / 256 and a group per 32 of the rest, stays on the device
-  const int64_t longest = ctx->n_pairs / (INV_LONG + 1) < n ? ctx->n_pairs / (INV_LONG + 1) : n;
-  const int64_t items = longest + (n - longest + 31) / 32 + 1;
+  // a warp per item; their number, one for each long particle and one for 32 of
+  // the rest, stays on the device
+  const int64_t longest = ctx->inv_longest, items = longest + (n - longest + 31) / 32 + 1;
   inv_apply<<<nblk(items * 32, INV_THREADS), INV_THREADS, 0, s>>>(n, ctx->inv_nlong, ctx->inv_order, ctx->inv_pid,
                                                                   ctx->inv_off, ctx->inv_base, ctx->inv_cell,
                                                                   ctx->inv_frac, cv, particle_value);
