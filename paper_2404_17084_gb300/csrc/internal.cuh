@@ -160,7 +160,7 @@ struct map_ctx {
   DevBuf ws_misc[8];
   DevBuf ws_grid[4];                   // grid preparation: face -> cell, per-face volume term and radius^2,
                                        // FP32 vertex copies
-  DevBuf ws_vor[23];                   // grid construction: buckets, cell slots, CSR arrays
+  DevBuf ws_vor[22];                   // grid construction: buckets, cell slots, CSR arrays
   DevBuf ws_inv[15];                   // particle-major copy of the pair list (inverse mapping, Eq. 4)
   DevBuf cub_tmp;
   bool rows_done = false;              // ws_pairs[8], the pair walk's rows, holds nothing a later step reads

@@ -979,8 +979,8 @@ int vor_buckets(map_ctx* ctx, const double* x, const double* y, const double* z,
   CUDA_TRY(cub::DeviceRadixSort::SortPairs(ctx->cub_tmp.p, tb, key, key_s, idx, idx_s, n, 0, bits, s));
   vor_bucket_bounds<<<nblk(n + 1, 256), 256, 0, s>>>(n, nb, key_s, off); ++ctx->launches;
   CUDA_TRY(cudaGetLastError());
-  float4 *hi, *lo;
-  MAP_TRY(ensure_t(ctx, ctx->ws_vor[22], 2 * n, &hi));
+  float4 *hi, *lo;  // (in the place of the grid's face planes, written last)
+  MAP_TRY(ensure_t(ctx, ctx->ws_vor[19], 2 * n, &hi));
   lo = hi + n;
   vor_split<<<nblk(n, 256), 256, 0, s>>>(n, x, y, z, idx_s, hi, lo); ++ctx->launches;
   CUDA_TRY(cudaGetLastError());

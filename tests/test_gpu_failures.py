@@ -119,9 +119,9 @@ def test_budget_below_one_request(small):
 # hbm_budget in MiB that holds it: half a percent above the least of the
 # library's first level-by-level octree and two-pass walk
 BUDGETS = [("solve_h", 2000, 1, 1, 0.489), ("map", 2000, 1, 1, 19.08), ("map", 2000, 1, 0, 24.39),
-           ("inverse", 2000, 1, 1, 29.6), ("pseudo", 2000, 1, 1, 0.581), ("solve_h", 60013, 1, 0, 12.34),
-           ("map", 60013, 30, 1, 38.12), ("inverse", 60013, 30, 1, 75.06), ("inverse", 60013, 30, 0, 80.56),
-           ("pseudo", 60013, 1, 1, 14.16)]
+           ("inverse", 2000, 1, 1, 29.6), ("pseudo", 2000, 1, 1, 0.581), ("grid", 2000, 1, 1, 23.76),
+           ("solve_h", 60013, 1, 0, 12.34), ("map", 60013, 30, 1, 38.12), ("inverse", 60013, 30, 1, 75.06),
+           ("inverse", 60013, 30, 0, 80.56), ("pseudo", 60013, 1, 1, 14.16), ("grid", 60013, 1, 1, 746.4)]
 
 
 @pytest.mark.parametrize("call,n,per_cell,precision,mib", BUDGETS)
