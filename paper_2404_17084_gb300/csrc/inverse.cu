@@ -36,20 +36,17 @@ namespace {
 constexpr int INV_THREADS = 128;
 
 // the place of every particle on the curve (the tree's order; the particles' own
-// when there is none of this size)
+// when there is none of this size), and rank[morton[k]] = k, the Morton rank of
+// every cell
 __global__ void inv_places(int64_t n, const int32_t* __restrict__ idx, int32_t* __restrict__ place,
-                           int32_t* __restrict__ pid) {
+                           int32_t* __restrict__ pid, int64_t nc, const int32_t* __restrict__ morton,
+                           int32_t* __restrict__ rank) {
   const int64_t stride = (int64_t)gridDim.x * blockDim.x;
   for (int64_t k = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; k < n; k += stride) {
     const int32_t a = idx ? idx[k] : (int32_t)k;
     place[a] = (int32_t)k;
     pid[k] = a;
   }
-}
-
-// rank[morton[k]] = k: the Morton rank of every cell
-__global__ void inv_rank(int64_t nc, const int32_t* __restrict__ morton, int32_t* __restrict__ rank) {
-  const int64_t stride = (int64_t)gridDim.x * blockDim.x;
   for (int64_t k = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; k < nc; k += stride) rank[morton[k]] = (int32_t)k;
 }
 
@@ -88,7 +85,8 @@ __global__ void inv_bounds(int64_t np, int64_t n, const int32_t* __restrict__ ke
 }
 
 // The order of the work: first the particles of more than INV_LONG entries,
-// then windows of 2^INV_WINDOW places, by decreasing count within one.
+// then windows of 2^INV_WINDOW places, by decreasing count within one, to two
+// entries (8 bits of the sort's key: up to 2^17 particles sort in two passes).
 constexpr unsigned INV_LONG = 256;
 constexpr int INV_WINDOW = 10;
 
@@ -99,7 +97,7 @@ __global__ void inv_keys(int64_t n, int64_t long_above, const int64_t* __restric
   const int64_t stride = (int64_t)gridDim.x * blockDim.x;
   for (int64_t a = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; a < n; a += stride) {
     const int64_t c = ioff[a + 1] - ioff[a];
-    key[a] = c > long_above ? 0u : (uint32_t)(((a >> INV_WINDOW) + 1) << 9 | (int64_t)(INV_LONG - c));
+    key[a] = c > long_above ? 0u : (uint32_t)(((a >> INV_WINDOW) + 1) << 8 | (int64_t)((INV_LONG - c) >> 1));
     ids[a] = (int32_t)a;
     const unsigned here = __activemask(), m = __ballot_sync(here, c > long_above);
     if (m && (int)(threadIdx.x & 31) == __ffs(here) - 1) atomicAdd(nlong, (unsigned long long)__popc(m));
@@ -108,17 +106,17 @@ __global__ void inv_keys(int64_t n, int64_t long_above, const int64_t* __restric
 
 // Work items: one per long particle, its entries contiguous, then one per 32
 // others in that order, interleaved up to the longest's count.  Items beyond
-// the last (of n + 1) are empty.
+// the last (up to room, for the most long particles there can be) are empty.
 __device__ __forceinline__ int64_t item_count(int64_t n, int64_t nlong) { return nlong + (n - nlong + 31) / 32; }
 
 // an item's entries, padding included (one warp per item)
-__global__ void inv_sizes(int64_t n, const int64_t* __restrict__ nlong_p, const int32_t* __restrict__ order,
+__global__ void inv_sizes(int64_t n, int64_t room, const int64_t* __restrict__ nlong_p, const int32_t* __restrict__ order,
                           const int64_t* __restrict__ ioff, int64_t* __restrict__ size) {
   const int lane = threadIdx.x & 31;
   const int64_t nw = ((int64_t)gridDim.x * blockDim.x) >> 5, nlong = *nlong_p, items = item_count(n, nlong);
-  for (int64_t it = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5; it <= n; it += nw) {
+  for (int64_t it = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5; it < room; it += nw) {
     if (it >= items) {  // nothing from here on: 32 places at a time
-      for (int64_t k = it + (int64_t)lane * nw; k <= n; k += 32 * nw) size[k] = 0;
+      for (int64_t k = it + (int64_t)lane * nw; k < room; k += 32 * nw) size[k] = 0;
       return;
     }
     const int64_t k = it < nlong ? it : nlong + 32 * (it - nlong) + lane;
@@ -249,14 +247,24 @@ int build_index(map_ctx* ctx, cudaStream_t s, bool groups) {
   int32_t *place, *pid;
   MAP_TRY(ensure_t(ctx, ctx->ws_inv[6], n, &place));
   MAP_TRY(ensure_t(ctx, ctx->ws_inv[13], n, &pid));
-  inv_places<<<g, 256, 0, s>>>(n, ctx->tree.n == n ? ctx->tree.idx : nullptr, place, pid); ++ctx->launches;
+  // the pair walk's Morton order of the cells, sorted by pairs_build with the
+  // list this copy is made from (a buffer no other step writes)
+  int32_t* rank = nullptr;
+  if (np > 0) {
+    if (ctx->ws_pairs[14].cap < (size_t)nc * sizeof(int32_t)) return MAP_EINVAL;
+    ctx->inv_morton = static_cast<const int32_t*>(ctx->ws_pairs[14].p);
+    MAP_TRY(ensure_t(ctx, ctx->ws_inv[11], nc, &rank));
+  }
+  inv_places<<<g, 256, 0, s>>>(n, ctx->tree.n == n ? ctx->tree.idx : nullptr, place, pid, np > 0 ? nc : 0,
+                               ctx->inv_morton, rank);
+  ++ctx->launches;
   CUDA_TRY(cudaGetLastError());
   ctx->inv_pid = pid;
-  // A window's groups, by decreasing count, are padded by at most 32 x (its
-  // largest - its smallest count), the group that crosses into the next window
-  // by 32 x 256, the last one by its missing lanes: 16 entries per particle and
-  // 3 x 8192 hold them all.
-  const int64_t room = groups ? np + 16 * n + 3 * 8192 : np;
+  // A window's groups, by decreasing count to two entries, are padded by at most
+  // 32 x (its largest - its smallest count + a 1 for each of 33 groups), the group
+  // that crosses into the next window by 32 x 256, the last one by its missing
+  // lanes: 18 entries per particle and 4 x 8192 hold them all.
+  const int64_t room = groups ? np + 18 * n + 4 * 8192 : np;
   // (the particles of more than INV_LONG entries: at most np / (INV_LONG + 1))
   const int64_t longest = groups && np / (INV_LONG + 1) < n ? np / (INV_LONG + 1) : n;
   unsigned long long* val_s = nullptr;
@@ -267,15 +275,6 @@ int build_index(map_ctx* ctx, cudaStream_t s, bool groups) {
     MAP_TRY(ensure_t(ctx, ctx->ws_inv[2], room, &val));
     MAP_TRY(ensure_t(ctx, ctx->ws_inv[3], np, &val_s));
     MAP_TRY(ensure_t(ctx, ctx->ws_inv[4], np, &key_s));
-    // the pair walk's Morton order of the cells, sorted by pairs_build with
-    // the list this copy is made from (a buffer no other step writes)
-    if (ctx->ws_pairs[14].cap < (size_t)nc * sizeof(int32_t)) return MAP_EINVAL;
-    const int32_t* morton = static_cast<const int32_t*>(ctx->ws_pairs[14].p);
-    int32_t* rank;
-    MAP_TRY(ensure_t(ctx, ctx->ws_inv[11], nc, &rank));
-    inv_rank<<<g, 256, 0, s>>>(nc, morton, rank); ++ctx->launches;
-    CUDA_TRY(cudaGetLastError());
-    ctx->inv_morton = morton;
     inv_pack<<<g, 256, 0, s>>>(nc, ctx->pair_off, ctx->pair_idx, place, rank, key, val); ++ctx->launches;
     CUDA_TRY(cudaGetLastError());
     size_t tb = 0;
@@ -303,22 +302,23 @@ int build_index(map_ctx* ctx, cudaStream_t s, bool groups) {
   ++ctx->launches;
   CUDA_TRY(cudaGetLastError());
   size_t tb2 = 0;
-  const int cb = bits_for(((n >> INV_WINDOW) + 2) << 9);
+  const int cb = bits_for(((n >> INV_WINDOW) + 2) << 8);
   CUDA_TRY(cub::DeviceRadixSort::SortPairs(nullptr, tb2, okey, okey_s, ids, order, n, 0, cb, s));
   MAP_TRY(ctx_ensure(ctx, ctx->cub_tmp, tb2));
   CUDA_TRY(cub::DeviceRadixSort::SortPairs(ctx->cub_tmp.p, tb2, okey, okey_s, ids, order, n, 0, cb, s));
   if (np > 0) {
     int32_t* cell = static_cast<int32_t*>(ctx->ws_inv[1].p);
     double* f = static_cast<double*>(ctx->ws_inv[2].p);
+    const int64_t items = longest + (n - longest + 31) / 32 + 1;
     int64_t *size, *base;
-    MAP_TRY(ensure_t(ctx, ctx->ws_inv[14], 2 * (n + 2), &size));
-    base = size + (n + 2);
-    inv_sizes<<<g, 256, 0, s>>>(n, nlong, order, ioff, size); ++ctx->launches;
+    MAP_TRY(ensure_t(ctx, ctx->ws_inv[14], 2 * items, &size));
+    base = size + items;
+    inv_sizes<<<g, 256, 0, s>>>(n, items, nlong, order, ioff, size); ++ctx->launches;
     CUDA_TRY(cudaGetLastError());
     size_t tb = 0;
-    CUDA_TRY(cub::DeviceScan::ExclusiveSum(nullptr, tb, size, base, n + 1, s));
+    CUDA_TRY(cub::DeviceScan::ExclusiveSum(nullptr, tb, size, base, items, s));
     MAP_TRY(ctx_ensure(ctx, ctx->cub_tmp, tb));
-    CUDA_TRY(cub::DeviceScan::ExclusiveSum(ctx->cub_tmp.p, tb, size, base, n + 1, s));
+    CUDA_TRY(cub::DeviceScan::ExclusiveSum(ctx->cub_tmp.p, tb, size, base, items, s));
     inv_fill<<<g, 256, 0, s>>>(n, nlong, order, ioff, base, val_s, ctx->pair_frac, cell, f); ++ctx->launches;
     CUDA_TRY(cudaGetLastError());
     ctx->inv_cell = cell;
