@@ -102,6 +102,27 @@ DM_FN double root(double x) {
   return g;
 }
 
+// a / b, |a| < |b|, normal: both scaled by b's exponent (integer operations),
+// then an FP32 quotient and two corrections by exact residuals (2^-54 of 1).
+DM_FN double quot(double a, double b) {
+  const int64_t sh = (int64_t)(0x3ff00000 - (hi32(b) & 0x7ff00000)) << 32;
+  const double A = from_bits(bits(a) + sh), B = from_bits(bits(b) + sh);
+  const float r = rcp_seed(f32(B));
+  double v = f64(f32(A) * r);
+  v += f64(f32(fma(-B, v, A)) * r);
+  v += f64(f32(fma(-B, v, A)) * r);
+  return v;
+}
+// the length of a squared length d2 < 1e30, and 1 / len, len < 1e15
+DM_FN double length(double d2) { return d2 > 1e-20 ? root(d2) : sqrt(d2); }
+DM_FN double inverse(double len) {
+  const float r = rcp_seed(f32(len));
+  double v = f64(r);
+  v += f64(f32(fma(-len, v, 1.0)) * r);
+  v += f64(f32(fma(-len, v, 1.0)) * r);
+  return len > 1e-18 ? v : 1.0 / len;
+}
+
 // Tables of atan(i / 512), i = 0..512, and of c and -ln c for the 512
 // intervals of [1, 2): c = the reciprocal of an interval's middle.
 constexpr int TAB = 512;

@@ -222,22 +222,6 @@ __device__ __forceinline__ double dist2(double ex, double ey, double ez) {
   return __fma_rn(ez, ez, __fma_rn(ey, ey, __dmul_rn(ex, ex)));
 }
 
-// a / b, |a| < |b|: an FP32 quotient and two corrections by exact residuals
-__device__ __forceinline__ double quot(double a, double b) {
-  const float r = dm::rcp_seed(dm::f32(b));
-  double v = dm::f64(dm::f32(a) * r);
-  v += dm::f64(dm::f32(fma(-b, v, a)) * r);
-  v += dm::f64(dm::f32(fma(-b, v, a)) * r);
-  return v;
-}
-__device__ __forceinline__ double length(double d2) { return d2 > 1e-20 ? dm::root(d2) : sqrt(d2); }
-__device__ __forceinline__ double inverse(double len) {
-  const float r = dm::rcp_seed(dm::f32(len));
-  double v = dm::f64(r);
-  v += dm::f64(dm::f32(fma(-len, v, 1.0)) * r);
-  v += dm::f64(dm::f32(fma(-len, v, 1.0)) * r);
-  return len > 1e-18 ? v : 1.0 / len;
-}
 __device__ __forceinline__ float rmax_of(double rmax2) { return sqrtf(dm::f32(rmax2)); }
 __device__ __forceinline__ float4 f32_of(double x, double y, double z) {
   return make_float4(dm::f32(x), dm::f32(y), dm::f32(z), 0.f);
@@ -367,7 +351,7 @@ __device__ __noinline__ int cell_clip(CellWarp& W, double nx, double ny, double 
     const int id = nv + __popc(mf & lt);
     if (nv + __popc(mf) > VOR_MAXV) return -1;
     if (on && first == k) {
-      const double sa = W.s[a], t = quot(sa, sa - W.s[c]);
+      const double sa = W.s[a], t = dm::quot(sa, sa - W.s[c]);
       const double xa = W.x[b][a], ya = W.y[b][a], za = W.z[b][a];
       const double x = fma(W.x[b][c] - xa, t, xa), y = fma(W.y[b][c] - ya, t, ya), z = fma(W.z[b][c] - za, t, za);
       const double r = dist2(x, y, z);
@@ -743,8 +727,8 @@ __global__ void __launch_bounds__(VW * 32) vor_cells(int64_t n, const double* __
   {
     double nx = 0, ny = 0, nz = 0, len = 0;
     if (lane < kn) {
-      len = length(kd);
-      const double il = inverse(len);
+      len = dm::length(kd);
+      const double il = dm::inverse(len);
       nx = (x[kj] - sx) * il; ny = (y[kj] - sy) * il; nz = (z[kj] - sz) * il;
     }
     const float fx = dm::f32(nx), fy = dm::f32(ny), fz = dm::f32(nz), fd = 0.5f * dm::f32(len);
@@ -830,7 +814,7 @@ __global__ void __launch_bounds__(VW * 32) vor_cells(int64_t n, const double* __
           const double e2 = dist2(ex, ey, ez);
           if (e2 <= 0.0 || e2 >= 4.0 * W.rmax2) continue;
           if (r <= 1 && (e2 < kth || (e2 == kth && jk <= __shfl_sync(VFULL, kj, 31)))) continue;  // in the list
-          const double len = length(e2), inv = inverse(len);
+          const double len = dm::length(e2), inv = dm::inverse(len);
           if (cell_clip(W, ex * inv, ey * inv, ez * inv, 0.5 * len, jk) < 0) { bad = true; break; }
         }
       }
