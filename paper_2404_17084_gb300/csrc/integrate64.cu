@@ -188,8 +188,11 @@ __device__ __forceinline__ void edge_round(DWarp& W, const dm::Tables* T, const 
   const double2 e01 = __ldg(E), e23 = __ldg(E + 1), e45 = __ldg(E + 2), e67 = __ldg(E + 3), e8_ = __ldg(E + 4);
   const double yx = W.py[0][o], yy = W.py[1][o], yz = W.py[2][o], hi_ = W.py[3][o];
   __syncwarp();  // the records are taken: new ones may overwrite them
-  // R0 = m.y - delta / h (> 0 inside) and the vertices' positions along the edge
-  const double R0s = fma(e01.x, yx, fma(e01.y, yy, fma(e23.x, yz, -(e23.y * hi_))));
+  // R0 = m.y - delta / h (> 0 inside) and the vertices' positions along the edge.
+  // Offsets over h stay unrounded here as in the planes' distances: the rounding
+  // of y is then one displacement of the particle for all of them, and one that
+  // lies on several planes to the last bit has the same side of each everywhere.
+  const double R0s = fma(-e23.y, hi_, fma(e01.x, yx, fma(e01.y, yy, e23.x * yz)));
   const double foot = fma(e45.x, yx, fma(e45.y, yy, e67.x * yz));
   const double aa = fma(e67.y, hi_, -foot), bb = fma(e8_.x, hi_, -foot);
   const bool ein = !dm::sign(R0s) || R0s == 0.0;
@@ -320,10 +323,7 @@ __global__ void __launch_bounds__(DW * 32, DCTA) pair_integrals_fp64(BatchArgs B
         const double4_32a F = staged ? W.fpl[fi] : A.face64[f0 + fi];
         const float4 Q = staged ? W.fsp[fi] : A.fsph[f0 + fi];
         const int ke = staged ? W.fend[fi] : (int)(A.fvo[f0 + fi + 1] - l0);
-        // (the product rounded by itself, as y is: a particle on the plane to the
-        // last bit gets 0 and is moved inside with the faces beside it; fused, it
-        // got the rounding of y and a side of its own on each face)
-        const double r0s = __dsub_rn(__dmul_rn(F.w, hinv), fma(F.x, yx, fma(F.y, yy, F.z * yz)));
+        const double r0s = fma(F.w, hinv, -fma(F.x, yx, fma(F.y, yy, F.z * yz)));
         const bool fin = !dm::sign(r0s) || r0s == 0.0;
         const double r0 = dm::max2(dm::abs2(r0s), EPS);
         if (COUNT && active) wc.faces++;

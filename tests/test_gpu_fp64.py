@@ -81,3 +81,26 @@ def test_small_particles_at_small_faces():
     p = synth.Particles(*(np.ascontiguousarray(at[:, k]) for k in range(3)), np.full(len(at), 1.0 / len(at)))
     got = gpu_map(g, p, np.full(len(at), h), 0)
     assert np.max(np.abs(np.bincount(got["idx"], got["frac"], len(at)) - 1.0)) < 1e-4
+
+
+@pytest.mark.parametrize("h,most,tol", [(0.02, 2, 1e-11), (1e-4, 2, 1e-11), (1e-8, 3, 1e-7), (1e-10, 3, 1e-5)])
+def test_particles_on_a_cubic_grid(h, most, tol):
+    """The faces and edges of cells of a sixth, whose planes are no binary
+    fractions, and their corners at sizes where y's rounding, 1e-16 / h of the
+    cell, is more than the 1e-12 h of the displacement (it moves the fractions
+    by as much: tol)."""
+    product = lambda v: np.stack(np.meshgrid(*[v] * 3, indexing="ij"), -1).reshape(-1, 3)  # noqa: E731
+    g = synth.voronoi(product((np.arange(6) + 0.5) / 6))
+    for a in (g.vx, g.vy, g.vz, g.face_plane[:, 3]):
+        a[...] = np.round(a * 6) / 6
+    g.face_plane[:, :3] = np.round(g.face_plane[:, :3])
+    k = product(np.arange(1, 12))
+    k = k[np.sum(k % 2 == 0, axis=1) <= most]
+    at = k / 12.0
+    p = synth.Particles(*(np.ascontiguousarray(at[:, i]) for i in range(3)), np.full(len(at), 1.0 / len(at)))
+    got = gpu_map(g, p, np.full(len(at), h), 0)
+    cell = np.repeat(np.arange(g.ncell), np.diff(got["off"]))
+    near = np.max(np.abs(at[got["idx"]] - g.site[cell]), axis=1) < 0.084
+    want = np.where(near, 0.5 ** np.sum(k % 2 == 0, axis=1)[got["idx"]], 0.0)
+    assert np.allclose(np.bincount(got["idx"], want), 1.0)
+    assert np.max(np.abs(got["frac"] - want)) < tol
