@@ -163,6 +163,7 @@ struct map_ctx {
   DevBuf ws_vor[22];                   // grid construction: buckets, cell slots, CSR arrays
   DevBuf ws_inv[15];                   // particle-major copy of the pair list (inverse mapping, Eq. 4)
   DevBuf cub_tmp;
+  int64_t no_pool_from = INT64_MAX;    // cells from which the budget did not hold the pair walk's pool
   bool rows_done = false;              // ws_pairs[8], the pair walk's rows, holds nothing a later step reads
   DevTree tree;
   int64_t node_cap0 = 0;  // > 0: octree node arrays start at this capacity (a context whose workspace is fixed)

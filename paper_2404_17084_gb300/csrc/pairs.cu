@@ -802,18 +802,22 @@ int walk_to_list(map_ctx* ctx, const PreparedGrid* g, cudaStream_t s, const Pair
   return walk_list(ctx, P, nc, *off, *list, read ? INT64_MAX : np, s);
 }
 
-// The same, without the pool when the budget does not hold it.
+// The same, without the pool when the budget does not hold it: later calls on
+// as many cells do not try it again, which would walk twice on each.
 int build_list(map_ctx* ctx, const PreparedGrid* g, cudaStream_t s, const PairBufs& out, int64_t& np, int64_t** off,
                int32_t** list) {
   const int64_t np0 = np;
-  const int r = walk_to_list(ctx, g, s, out, true, np, off, list);
-  if (r != MAP_ENOMEM) return r;
+  const bool pool = g->ncell < ctx->no_pool_from;
+  const int r = walk_to_list(ctx, g, s, out, pool, np, off, list);
+  if (r != MAP_ENOMEM || !pool) return r;
   DevBuf& rows = ctx->ws_pairs[8];
   dev_free(ctx, rows.p);
   ctx->bytes_in_use -= rows.cap;
   rows = DevBuf();
   np = np0;
-  return walk_to_list(ctx, g, s, out, false, np, off, list);
+  MAP_TRY(walk_to_list(ctx, g, s, out, false, np, off, list));
+  ctx->no_pool_from = g->ncell;
+  return MAP_OK;
 }
 
 }  // namespace

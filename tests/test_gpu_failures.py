@@ -163,3 +163,31 @@ def test_budgets_that_held_a_call_still_do(call, n, per_cell, precision, mib):
             L.map_destroy(ctx)
     for a, b in zip(*out):
         assert torch.equal(a, b)
+
+
+@pytest.mark.parametrize("precision,mib", [(1, 19.08), (0, 24.39)])
+def test_a_tight_budget_walks_once_per_call(precision, mib):
+    """A call whose budget did not hold the pair walk's pool leaves it out of
+    the next ones, which launch as much as without a budget."""
+    L = lib()
+    p = synth.lognormal_particles(2000, 3, ngrid=64)
+    grid = synth.voronoi(p.pos())
+    x, y, z, m, h = dev_particles(p)
+    hctx = L.map_init(L.map_config_default(precision=1))
+    L.solve_h(hctx, L.make_particles(x, y, z, None, h))
+    L.map_destroy(hctx)
+    n = []
+    for budget in (0, int(mib * 2 ** 20)):
+        ctx = L.map_init(L.map_config_default(precision=precision, hbm_budget=budget))
+        try:
+            hd = L.map_grid_upload(ctx, L.grid_to_device(grid))
+            mass = torch.empty(grid.ncell, dtype=torch.float64, device="cuda")
+            at = []
+            for _ in range(3):
+                L.map_particles_to_cells(ctx, L.make_particles(x, y, z, m, h), hd, mass)
+                at.append(L.map_get_work(ctx)[1])
+            n.append((at[0], at[1] - at[0], at[2] - at[1]))
+        finally:
+            L.map_destroy(ctx)
+    print(n)
+    assert n[1][1:] == n[0][1:]
