@@ -254,13 +254,15 @@ int map_copy_pairs(map_ctx* ctx, int64_t* pair_off, int32_t* pair_idx, double* p
  * list gets 0.
  *
  * The first call after a mapping builds a particle-major copy of its pair
- * list (cell and f_ai of every pair, 12 bytes per pair, and padding of at most
- * 16 pairs per particle, plus 48 bytes per particle and 12 per cell), kept by
- * the context until the next mapping call; later calls with other cell
- * values reuse it.  The build's sort workspace (about 12 bytes per pair) also
- * stays with the context, for the next mapping's build, until map_destroy.
- * Asynchronous on stream (ordered after the mapping call like every call of
- * the context).
+ * list (cell and f_ai of every pair, 12 bytes per pair, with padding of at
+ * most 18 pairs per particle and 32768 more; some 30 bytes per particle and 12
+ * per cell), kept by the context until the next mapping call; later calls
+ * with other cell values reuse it.  The build's sort workspace (about 24 bytes
+ * per pair, the library sort's own included) also stays with the context, for
+ * the next mapping's build, until map_destroy.  All have a quarter's room to
+ * grow.  Where an hbm_budget does not hold the padding the copy is made
+ * without it (the same sums, slower).  Asynchronous on stream (ordered after
+ * the mapping call like every call of the context).
  * Errors: MAP_EINVAL (NULL pointer; no single mapping call with per-pair
  * integrals in this context: map_batch and the server keep none; n is not
  * that call's particle count; 2^32 or more pairs), MAP_ENOMEM, MAP_ECUDA. */
@@ -442,7 +444,12 @@ void map_server_destroy(map_server* srv);
 /* Solve h_a = hfact * n_a(h_a)^(-1/3), n_a(h) = sum_b W(|r_a - r_b|, h)
  * (self term included) for every particle: Newton-Raphson (at most 30
  * iterations, converged at |dh|/h < 1e-10), else bisection on
- * [h0/16, 16 h0] (|dh|/h < 1e-12), else the estimate h0.  A MAP_MIXED
+ * [h0/16, 16 h0] (|dh|/h < 1e-12), else the estimate h0.  A MAP_FP64
+ * context lets FP32 sums lead to the root and ends with steps of third order
+ * on FP64 sums, until one is below 2e-6 of h (its cube is what is left); a
+ * particle whose FP32 solve comes near a decision, or does not settle, is
+ * solved by the rules above on FP64 sums throughout, so h and route are
+ * those of FP64 sums.  A MAP_MIXED
  * context sums the kernel in FP32 (on FP32 hi/lo splits of the coordinates),
  * in the bisection too, iterates Newton in FP32 (its converged step applied
  * in FP64) and stops it at |dh|/h < 1e-6, which gives h to ~1e-7 relative

@@ -61,7 +61,7 @@ constexpr int HS_PCAP = 512;   // one particle's own candidates (within 2.5 h of
 constexpr int HS_WIN = 8;      // sorted positions per warp, which takes the leaves that start among them: about
                                // one leaf (7 particles on average), so that a snapshot of 60,000 gives 7,500
                                // warps (32 positions: 1,875, one wave as long as its slowest four leaves)
-constexpr int HS_MLP = 2;      // candidates per lane in flight during a pass (4: more registers, 12.6 ms at 2^20)
+constexpr int HS_MLP = 2;      // candidates per lane in flight during a pass (4: more registers, 13.9 ms for 13.2 at 2^20)
 constexpr int HS_REG = 6;      // own candidates per lane held in registers (192 per particle; 113 on average)
 constexpr unsigned FULL = 0xffffffffu;
 
@@ -841,7 +841,7 @@ int h_solve_run(map_ctx* ctx, const double* x, const double* y, const double* z,
   // Candidates per lane in flight over a list that outgrew its buffer: a small
   // set lasts as long as the leaf with the longest list (60,013 particles: 2.24
   // ms with 4, 2.41 with 2; 262,144: 3.83, 4.31), a large one as long as its
-  // warps take together, and the registers of 4 cost it some (2^20: 11.3, 10.5).
+  // warps take together, and the registers of 4 cost it some (2^20: 13.7, 13.2).
   const bool mixed = ctx->cfg.precision != MAP_FP64;
   auto kern = n < (int64_t(1) << 19) ? (mixed ? h_solve_leaves<true, 4> : h_solve_leaves<false, 4>)
                                      : (mixed ? h_solve_leaves<true, 2> : h_solve_leaves<false, 2>);

@@ -9,6 +9,7 @@
 #include <cub/cub.cuh>
 
 #include "internal.cuh"
+#include "wedge.cuh"
 
 namespace {
 
@@ -19,8 +20,6 @@ struct PairTree {
   const int32_t* idx;
   const int64_t *nb, *ne, *fc;
   const int32_t* nch;
-  const unsigned long long* bbox;
-  const unsigned long long* hmax;
   const float* box32;  // outward-rounded FP32 boxes and largest h (8 floats per node)
 };
 
@@ -170,24 +169,9 @@ struct PairRows {
   unsigned long long* n_again;
 };
 
-// FP32 pairs in one instruction
-struct f2 { float x, y; };
-__device__ __forceinline__ unsigned long long f2_bits(f2 a) {
-  return (unsigned long long)__float_as_uint(a.x) | ((unsigned long long)__float_as_uint(a.y) << 32);
-}
-__device__ __forceinline__ f2 f2_from(unsigned long long b) {
-  return f2{__uint_as_float((unsigned)b), __uint_as_float((unsigned)(b >> 32))};
-}
-__device__ __forceinline__ f2 add2(f2 a, f2 b) {
-  unsigned long long d;
-  asm("add.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(f2_bits(a)), "l"(f2_bits(b)));
-  return f2_from(d);
-}
-__device__ __forceinline__ f2 mul2(f2 a, f2 b) {
-  unsigned long long d;
-  asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(f2_bits(a)), "l"(f2_bits(b)));
-  return f2_from(d);
-}
+using wedge::add2;
+using wedge::f2;
+using wedge::mul2;
 
 struct WalkWarp {
   int2 stk[PT_STK];       // internal node: (first child, children); leaf: (first position, -particles)
@@ -725,8 +709,7 @@ int walk_rows(map_ctx* ctx, const PreparedGrid* g, cudaStream_t s, PairWalk& P, 
   MAP_TRY(ctx_ensure(ctx, ctx->cub_tmp, tb));
   CUDA_TRY(cub::DeviceRadixSort::SortPairs(ctx->cub_tmp.p, tb, k_in, k_out, o_in, P.order, nc, 0, 30, s));
 
-  P.T = PairTree{T.xs, T.ys, T.zs, T.hs, T.hs32, T.split, T.idx, T.begin, T.end, T.first_child, T.nchild, T.bbox_bits,
-                 T.hmax_bits, T.box32};
+  P.T = PairTree{T.xs, T.ys, T.zs, T.hs, T.hs32, T.split, T.idx, T.begin, T.end, T.first_child, T.nchild, T.box32};
   P.G = PairGrid{g->cell_face_off, g->face_plane, g->face32, g->site, g->rad, g->rin};
   MAP_TRY(ensure_t(ctx, ctx->ws_pairs[0], nc + 1, &P.count));
   const int64_t npool = pool ? nc / 32 + (2 * nc < 4096 ? 2 * nc : 4096) : 0;

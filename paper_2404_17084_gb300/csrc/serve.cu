@@ -90,10 +90,10 @@ double ms_between(std::chrono::steady_clock::time_point a, std::chrono::steady_c
 }
 
 // Device bytes of a prepared grid (its copy of the CSR and the geometry the
-// precision keeps: 12 floats per loop entry for the mixed build, 12 doubles
+// precision keeps: 12 floats per loop entry for the mixed build, 10 doubles
 // for FP64), with 25% headroom.
 size_t grid_bytes(const map_request& r, int precision) {
-  const double loop = precision != MAP_FP64 ? 64.0 : 112.0;
+  const double loop = precision != MAP_FP64 ? 64.0 : 96.0;
   return (size_t)(1.25 * (96.0 * r.ncell + 146.0 * r.nface + loop * r.nloop + 48.0 * r.nvert));
 }
 

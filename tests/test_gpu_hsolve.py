@@ -6,7 +6,8 @@ import torch
 
 import oracle
 import synth
-from gpu_helpers import dev_particles, lib, oracle_h
+from gpu_helpers import lib
+from gpu_helpers import dev_particles, oracle_h
 
 pytestmark = pytest.mark.gpu
 
